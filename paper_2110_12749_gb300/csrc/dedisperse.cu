@@ -869,6 +869,8 @@ const TiledVariant kVariants[] = {
 };
 constexpr int kNumVariants = sizeof(kVariants) / sizeof(kVariants[0]);
 
+constexpr int kMmaVariant = kNumVariants;  // the tensor-core kernel (dd_mma.cu)
+
 constexpr int kDefaultVariant = 32;  // 15 DMs x 768 samples, 64-channel stages, precomputed lists
 
 // Variants tried in order when a plan is created; the first whose stages fit
@@ -882,7 +884,7 @@ constexpr int kDefaultVariant = 32;  // 15 DMs x 768 samples, 64-channel stages,
 const int kAutoList[] = {kDefaultVariant, 42, 34, 44, 40, 41};
 
 // Variants the batch autotuner times (those that fit the batch are timed).
-const int kTuneList[] = {kDefaultVariant, 42, 35, 31, 22, 43, 44, 36, 34, 40};
+const int kTuneList[] = {kMmaVariant, kDefaultVariant, 42, 35, 31, 22, 43, 44, 36, 34, 40};
 
 // Shared memory of one CTA: all of an SM's 227 KB, or half of it (less the
 // per-CTA reserve) for CTAs of at most 8 warps that run two per SM.
@@ -913,6 +915,23 @@ TileFit fit_variant(const TiledVariant &v, int64_t spread) {
 }
 
 bool lists_ok(const TiledVariant &v, bool have_lists) { return !v.pre || have_lists; }
+
+constexpr int kMmaMaxChannels = 65793;  // 255 nchan < 2^24: the FP32 sums are exact
+constexpr int kMmaMinTile = 256;        // shortest tile the tensor-core kernel is used at
+
+// Additions per clock and SM of the byte kernel's automatic variants (measured).
+double byte_rate(int variant) { return variant == kDefaultVariant ? 86.0 : (variant == 42 ? 78.0 : 60.0); }
+
+// Estimated SM clocks of a launch of one beam: waves of one CTA per SM, 13,000
+// clocks of prologue and epilogue per CTA (256 channels, 200 trials, 31,000 samples:
+// 186,000 measured, 188,000 estimated).
+double byte_launch_clocks(int variant, int nchan, int ndm, int64_t n_out, int num_sms) {
+    const TiledVariant &v = kVariants[variant];
+    const int t_eff = 128 * v.m - 4;
+    const int64_t items = (n_out + t_eff - 1) / t_eff * ((ndm + v.kdm - 1) / v.kdm);
+    return (double)((items + num_sms - 1) / num_sms) *
+           ((double)nchan * v.kdm * t_eff / byte_rate(variant) + 13000.0);
+}
 
 // The first variant of the automatic list that fits; -1 if none does.
 int choose_auto(const int64_t (&spread)[kNumKdm], const bool (&have_lists)[kNumCb]) {
@@ -1021,32 +1040,51 @@ bool plan_dedisperse_tiled(gsp_plan_s *p, TiledTables *tab) {
     // GSP_DD_VARIANT selects a tuning variant of the tiled kernel if it fits
     // this plan; otherwise the automatic choice.
     int variant = -1;
+    bool force_mma = false;
     if (const char *v = std::getenv("GSP_DD_VARIANT")) {
         const int k = std::atoi(v);
+        force_mma = k == kMmaVariant;
         if (k >= 0 && k < kNumVariants && lists_ok(kVariants[k], have_lists[cb_index(kVariants[k].cb)]) &&
             fit_variant(kVariants[k], g.spread[kdm_index(kVariants[k].kdm)]).ok)
             variant = k;
     }
+    const bool forced = variant >= 0;
     if (variant < 0) variant = choose_auto(g.spread, have_lists);
     if (variant < 0) {
         *tab = TiledTables();
         return false;
     }
-    const TiledVariant &v = kVariants[variant];
-    const TileFit f = fit_variant(v, g.spread[kdm_index(v.kdm)]);
-    g.kdm = v.kdm;
-    g.t_cta = 128 * v.m;
-    g.t_eff = 128 * v.m - 4;
-    g.cb = v.cb;
-    g.win = f.win;
-    g.stages = f.stages;
-    g.smem = f.smem;
-    g.ctas_per_sm = f.ctas_per_sm;
-    g.variant = variant;
+    // The tensor-core kernel where its time per addition on long inputs is estimated the
+    // smaller (measured, 4096 channels, 1000-1500 MHz, step 0.5: 135 additions per
+    // clock and SM against 86; step 1.5 or a 500-3300 MHz band, whose delays drift
+    // apart too fast: byte kernel).  A plan keeps its tables only if they may be used.
+    int byte_variant = -1;
+    if (C <= kMmaMaxChannels && mma_plan_tables(p->delays_h.data(), ndm, C,
+                                                !p->desc.freq_descending, &tab->mma)) {
+        MmaShape &m = p->mma.shape;
+        m.rmax = tab->mma.rmax;
+        m.mean_r = tab->mma.mean_cols_r;
+        m.frames_per_block = (double)tab->mma.frames.size() / (double)((ndm + 15) / 16);
+        const int T = mma_tile_len(m.rmax);
+        const double byte_clk = 16.0 * T * C / byte_rate(variant);
+        const double mma_clk = T >= kMmaMinTile ? mma_item_clocks(m, C, T) : 1e30;
+        if (force_mma && T >= 16) {
+            variant = kMmaVariant;
+        } else if (mma_clk > 1.2 * byte_clk) {
+            tab->mma = MmaTables();
+        } else if (!forced && mma_clk < byte_clk) {
+            byte_variant = variant;
+            variant = kMmaVariant;
+        }
+    } else {
+        tab->mma = MmaTables();
+    }
+    dedisperse_set_variant(p, variant);
+    g.byte_variant = byte_variant;
     return true;
 }
 
-int dedisperse_num_variants() { return kNumVariants; }
+int dedisperse_num_variants() { return kNumVariants + 1; }
 
 int dedisperse_tune_candidates(const int **list) {
     *list = kTuneList;
@@ -1060,7 +1098,8 @@ TileFit dedisperse_fit(int variant, const int64_t (&spread)[kNumKdm]) {
 }
 
 bool dedisperse_variant_usable(const gsp_plan_s *p, int variant) {
-    if (!p || p->simple_dd || variant < 0 || variant >= kNumVariants) return false;
+    if (!p || p->simple_dd || variant < 0 || variant > kMmaVariant) return false;
+    if (variant == kMmaVariant) return p->mma.d_frames != nullptr;
     const TiledVariant &v = kVariants[variant];
     const int o = kdm_index(v.kdm), ci = cb_index(v.cb);
     if (!p->d_blkmin[o] || !p->d_stspread[o][ci]) return false;
@@ -1069,6 +1108,18 @@ bool dedisperse_variant_usable(const gsp_plan_s *p, int variant) {
 }
 
 void dedisperse_set_variant(gsp_plan_s *p, int variant) {
+    if (variant == kMmaVariant) {
+        DDGeom &g = p->geom;
+        g.kdm = 16;
+        g.t_cta = mma_tile_len(p->mma.shape.rmax);
+        g.t_eff = kMmaMinBlock;  // search blocks at least this long have their sums fused
+        g.cb = 8;
+        g.win = g.stages = g.smem = 0;
+        g.ctas_per_sm = 1;
+        g.variant = variant;
+        g.byte_variant = -1;
+        return;
+    }
     const TiledVariant &v = kVariants[variant];
     const TileFit f = fit_variant(v, p->geom.spread[kdm_index(v.kdm)]);
     DDGeom &g = p->geom;
@@ -1081,6 +1132,7 @@ void dedisperse_set_variant(gsp_plan_s *p, int variant) {
     g.smem = f.smem;
     g.ctas_per_sm = f.ctas_per_sm;
     g.variant = variant;
+    g.byte_variant = -1;
 }
 
 int dedisperse_choose_variant(const gsp_plan_s *const *plans, int nplans) {
@@ -1096,7 +1148,8 @@ int dedisperse_choose_variant(const gsp_plan_s *const *plans, int nplans) {
     const int v0 = plans[0]->geom.variant;
     bool same = true;
     for (int i = 1; i < nplans; i++) same = same && plans[i]->geom.variant == v0;
-    if (same && lists_ok(kVariants[v0], have_lists[cb_index(kVariants[v0].cb)]) &&
+    if (same && v0 == kMmaVariant) return v0;
+    if (same && v0 < kNumVariants && lists_ok(kVariants[v0], have_lists[cb_index(kVariants[v0].cb)]) &&
         fit_variant(kVariants[v0], spread[kdm_index(kVariants[v0].kdm)]).ok)
         return v0;
     return choose_auto(spread, have_lists);
@@ -1105,8 +1158,19 @@ int dedisperse_choose_variant(const gsp_plan_s *const *plans, int nplans) {
 cudaError_t launch_dedisperse_batch(const BeamLaunch *beams, int nbeams, int variant,
                                     bool persistent, int num_sms, int *err, cudaStream_t s,
                                     int32_t *nlaunch) {
-    if (nbeams < 1 || nbeams > kMaxBatchBeams || variant < 0 || variant >= kNumVariants)
+    if (nbeams < 1 || nbeams > kMaxBatchBeams || variant < 0 || variant > kMmaVariant)
         return cudaErrorInvalidValue;
+    if (variant == kMmaVariant) {
+        // one short beam: the byte kernel where its waves are estimated to end earlier
+        const gsp_plan_s *p = beams[0].plan;
+        const int bv = p->geom.byte_variant;
+        int T = 0;
+        if (nbeams > 1 || bv < 0 ||
+            mma_launch_clocks(p->mma.shape, p->desc.nchan, p->desc.ndm, beams[0].n_out, num_sms, &T) <=
+                byte_launch_clocks(bv, p->desc.nchan, p->desc.ndm, beams[0].n_out, num_sms))
+            return launch_dedisperse_mma(beams, nbeams, num_sms, err, s, nlaunch);
+        variant = bv;
+    }
     const TiledVariant &v = kVariants[variant];
     const int o = kdm_index(v.kdm), ci = cb_index(v.cb);
     const int t_cta = 128 * v.m, t_eff = t_cta - 4;

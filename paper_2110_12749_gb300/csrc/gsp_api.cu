@@ -94,6 +94,12 @@ void free_plan(gsp_plan_s *p) {
     for (auto *b : p->d_fcnt) cudaFree(b);
     for (auto &row : p->d_stspread)
         for (auto *b : row) cudaFree(b);
+    cudaFree(p->mma.d_base);
+    cudaFree(p->mma.d_shift);
+    cudaFree(p->mma.d_frames);
+    cudaFree(p->mma.d_foff);
+    cudaFree(p->mma.d_crmax);
+    cudaFree(p->mma.d_rlast);
     cudaFree(p->d_err);
     cudaFree(p->d_prefix);
     cudaFree(p->d_order);
@@ -372,6 +378,15 @@ gsp_status gsp_plan_create(gsp_plan_t *out, const gsp_plan_desc *d) {
         if (st == GSP_OK && !tab.dpos[i].empty()) st = dalloc(&p->d_dpos[i], tab.dpos[i].size());
         if (st == GSP_OK && !tab.fcnt[i].empty()) st = dalloc(&p->d_fcnt[i], tab.fcnt[i].size());
     }
+    if (!tab.mma.frames.empty()) {
+        const gsp::MmaTables &m = tab.mma;
+        if (st == GSP_OK) st = dalloc(&p->mma.d_base, m.base.size());
+        if (st == GSP_OK) st = dalloc(&p->mma.d_shift, m.shift.size());
+        if (st == GSP_OK) st = dalloc(&p->mma.d_frames, m.frames.size());
+        if (st == GSP_OK) st = dalloc(&p->mma.d_foff, m.foff.size());
+        if (st == GSP_OK) st = dalloc(&p->mma.d_crmax, m.crmax.size());
+        if (st == GSP_OK) st = dalloc(&p->mma.d_rlast, m.rlast.size());
+    }
     if (st == GSP_OK) st = dalloc(&p->d_sigma_b, rows_blocks);
     if (st == GSP_OK) st = dalloc(&p->d_bad, rows_blocks);
     if (st == GSP_OK) st = dalloc(&p->d_bparam, rows_blocks);
@@ -403,6 +418,15 @@ gsp_status gsp_plan_create(gsp_plan_t *out, const gsp_plan_desc *d) {
     for (int i = 0; i < gsp::kNumCb; i++) {
         up(p->d_dpos[i], tab.dpos[i].data(), tab.dpos[i].size() * sizeof(int32_t));
         up(p->d_fcnt[i], tab.fcnt[i].data(), tab.fcnt[i].size() * sizeof(uint32_t));
+    }
+    if (!tab.mma.frames.empty()) {
+        const gsp::MmaTables &m = tab.mma;
+        up(p->mma.d_base, m.base.data(), m.base.size() * sizeof(int32_t));
+        up(p->mma.d_shift, m.shift.data(), m.shift.size());
+        up(p->mma.d_frames, m.frames.data(), m.frames.size() * sizeof(gsp::MmaFrame));
+        up(p->mma.d_foff, m.foff.data(), m.foff.size() * sizeof(int32_t));
+        up(p->mma.d_crmax, m.crmax.data(), m.crmax.size() * sizeof(int32_t));
+        up(p->mma.d_rlast, m.rlast.data(), m.rlast.size() * sizeof(int32_t));
     }
     if (e == cudaSuccess) e = cudaMemset(p->d_ncand, 0, sizeof(unsigned long long));
     if (e == cudaSuccess) e = cudaMemset(p->d_err, 0, sizeof(int));

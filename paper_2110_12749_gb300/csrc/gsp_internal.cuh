@@ -6,6 +6,7 @@
 #include <cstdint>
 #include <vector>
 
+#include "dd_mma.cuh"
 #include "gsp.h"
 
 namespace gsp {
@@ -58,6 +59,9 @@ struct DDGeom {
     int grp[kNumKdm] = {1, 1, 1};      // DM blocks per launch group
     int64_t spread[kNumKdm] = {};      // largest delay spread inside a DM block
     int variant = 0;   // template variant index
+    // the plan's choice by estimate was the tensor-core kernel: a launch takes this byte
+    // variant instead where it is estimated the faster (-1: the variant is fixed)
+    int byte_variant = -1;
 };
 
 // Launch geometry of one tile variant for a given largest in-block delay
@@ -69,6 +73,18 @@ struct TileFit {
     int stages = 0;
     int smem = 0;
     int ctas_per_sm = 1;
+};
+
+// Device tables of the tensor-core dedispersion kernel (see MmaTables), null
+// when the plan does not keep them.
+struct MmaDevice {
+    int32_t *d_base = nullptr;
+    uint8_t *d_shift = nullptr;
+    MmaFrame *d_frames = nullptr;
+    int32_t *d_foff = nullptr;
+    int32_t *d_crmax = nullptr;
+    int32_t *d_rlast = nullptr;
+    MmaShape shape;
 };
 
 }  // namespace gsp
@@ -112,6 +128,7 @@ struct gsp_plan_s {
     int64_t nb_max = 0;
 
     gsp::DDGeom geom;
+    gsp::MmaDevice mma;
 
     cudaEvent_t ev[3] = {nullptr, nullptr, nullptr};
     // host-input pipeline (gsp_search_host): copy stream and its events, created on first use
@@ -166,6 +183,9 @@ struct BeamLaunch {
 cudaError_t launch_dedisperse_batch(const BeamLaunch *beams, int nbeams, int variant,
                                     bool persistent, int num_sms, int *err, cudaStream_t s,
                                     int32_t *nlaunch);
+// The same on the tensor cores (plans that keep the MmaDevice tables).
+cudaError_t launch_dedisperse_mma(const BeamLaunch *beams, int nbeams, int num_sms, int *err,
+                                  cudaStream_t s, int32_t *nlaunch);
 int dedisperse_num_variants();
 // Variants the batch autotuner may time, in order of preference.
 int dedisperse_tune_candidates(const int **list);
@@ -234,6 +254,7 @@ struct TiledTables {
     std::vector<int32_t> dpos[kNumCb];
     std::vector<uint32_t> fcnt[kNumCb];
     std::vector<int32_t> stspread[kNumKdm][kNumCb];
+    MmaTables mma;  // empty frames: the plan does without the tensor-core kernel
 };
 // DM-block tables and per-stage spreads of every block size and stage width,
 // then the plan's variant and geometry.  Returns false (the plan then uses
