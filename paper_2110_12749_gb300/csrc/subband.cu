@@ -23,6 +23,7 @@
 #include <new>
 #include <vector>
 
+#include "dd_tiled.cuh"
 #include "gsp_internal.cuh"
 
 namespace {
@@ -132,67 +133,155 @@ __global__ void __launch_bounds__(256) downsample_pow2_kernel(const uint8_t *__r
 
 // ---------------------------------------------------------------------------
 // Stage 2 of sub-band dedispersion.  One CTA per (group g, 1024 output
-// samples); thread i owns outputs t0 + i + 256 j (j < 4) of every trial of
-// the group.  The group's rows S[s][g][t0 + min2[g][s] .. + 1024 + spread)
-// are staged in shared memory a chunk of sub-bands at a time, so the rows
-// are read from L2 once per group instead of once per trial; a trial then
-// reads its row at the offset off2[d][s] = d2[d][s] - min2[g][s].
+// samples): the group's rows S[s][g][t0 + min2[g][s] .. + 1024 + spread) are
+// read once per group and summed by each of its trials at the offset
+// d2[d][s] - min2[g][s].
+//
+// A producer warp copies the rows (1-D bulk copies, from the 16-byte boundary
+// below their start) into a ring of shared-memory stages of kS2Rows rows, with
+// full / empty mbarriers; eight consumer warps take trials w and w + 8, all 1024
+// samples each (32 per lane), so that a (row, trial) costs one offset for 32
+// conflict-free loads, and two rows share each three-input add.  Bound by the shared
+// loads, 32 additions per clock and SM: 2.75e10 additions (64 sub-bands, 2000
+// trials, 2^18-sample chunk) 11.2 -> 3.4 ms against the kernel that gave every
+// thread four samples of all 16 trials (one offset load per four additions, no
+// copies under the sums).
+// Every wait is bounded; a warp that gives up reports it and leaves, the producer only
+// after its copies have landed.
 constexpr int kMaxGroup = 16;
-constexpr int kS2Threads = 256;
-constexpr int kS2Tile = 4 * kS2Threads;
+constexpr int kS2Warps = 8;
+constexpr int kS2Tile = 1024;
+constexpr int kS2Rows = 4;                 // rows per stage
+constexpr long long kS2Budget = 2000000000ll;  // ~1 s of SM clock per wait
 
-__global__ void __launch_bounds__(kS2Threads) subband_sum_kernel(
-    const int32_t *__restrict__ S, int64_t s_stride, int nsdm, int nsub, int64_t n1,
+namespace ptx = gsp::ptx;
+
+__global__ void __launch_bounds__((kS2Warps + 1) * 32, 2) subband_sum_kernel(
+    const int32_t *__restrict__ S, int64_t s_stride, int nsdm, int nsub,
     const int32_t *__restrict__ min2, const int32_t *__restrict__ off2, int ndm, int group,
-    int row_len, int chunk, int64_t n_out, int32_t *__restrict__ D, int64_t d_stride) {
-    extern __shared__ __align__(16) int32_t sm[];
-    int32_t *soff = sm;                         // [group][nsub] offsets of the group's trials
-    int32_t *rows = sm + kMaxGroup * nsub;      // [chunk][row_len]
+    int pitch, int rows, int stages, int64_t n_out, int32_t *__restrict__ D, int64_t d_stride, int *err) {
+    extern __shared__ __align__(128) int32_t sm[];  // [stages][rows][pitch], then the barriers
+    const uint32_t sm0 = ptx::smem_addr(sm);
+    const uint32_t stage_bytes = (uint32_t)(rows * pitch * 4);
+    const uint32_t bar0 = sm0 + (uint32_t)stages * stage_bytes;
+    auto full = [&](int i) { return bar0 + 8u * (uint32_t)i; };
+    auto empty = [&](int i) { return bar0 + 8u * (uint32_t)(stages + i); };
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int g = blockIdx.y;
     const int64_t t0 = (int64_t)blockIdx.x * kS2Tile;
-    const int d0 = g * group;
-    const int gcount = min(group, ndm - d0);
-    for (int i = threadIdx.x; i < gcount * nsub; i += kS2Threads)
-        soff[i] = off2[(int64_t)d0 * nsub + i];
-    int32_t acc[kMaxGroup][4];
-#pragma unroll
-    for (int i = 0; i < kMaxGroup; i++)
-#pragma unroll
-        for (int j = 0; j < 4; j++) acc[i][j] = 0;
-    for (int s0 = 0; s0 < nsub; s0 += chunk) {
-        const int sc = min(chunk, nsub - s0);
-        __syncthreads();  // previous chunk consumed (and soff written)
-        for (int r = 0; r < sc; r++) {
-            const int s = s0 + r;
-            const int64_t base = t0 + min2[(int64_t)g * nsub + s];
-            const int32_t *src = S + ((int64_t)s * nsdm + g) * s_stride;
-            int32_t *dst = rows + r * row_len;
-            for (int i = threadIdx.x; i < row_len; i += kS2Threads) {
-                const int64_t t = base + i;
-                dst[i] = t < n1 ? __ldg(src + t) : 0;
+    const int nst = (nsub + rows - 1) / rows;
+    if (threadIdx.x == 0) {
+        for (int i = 0; i < stages; i++) {
+            ptx::mbar_init(full(i), 1);
+            ptx::mbar_init(empty(i), kS2Warps);
+        }
+        ptx::fence_barrier_init();
+    }
+    __syncthreads();
+    if (warp == kS2Warps) {
+        int slot = 0;
+        uint32_t par = 1;  // a fresh barrier's previous phase counts as complete
+        int issued = 0;
+        bool ok = true;
+        for (int st = 0; st < nst; st++) {
+            const int s = st * rows + lane;
+            const bool in = lane < rows && s < nsub;
+            int64_t a0 = 0;
+            uint32_t bytes = 0;
+            if (in) {
+                a0 = (t0 + __ldg(min2 + (int64_t)g * nsub + s)) & ~(int64_t)3;
+                bytes = 4u * (uint32_t)max((int64_t)0, min((int64_t)pitch, s_stride - a0));
+            }
+            const uint32_t tot = __reduce_add_sync(0xffffffffu, bytes);
+            if (!__all_sync(0xffffffffu, ptx::mbar_wait(empty(slot), par, kS2Budget))) {
+                ok = false;
+                break;
+            }
+            if (lane == 0) ptx::mbar_arrive_expect_tx(full(slot), tot);
+            __syncwarp();
+            if (bytes > 0)
+                ptx::bulk_g2s(sm0 + (uint32_t)slot * stage_bytes + (uint32_t)(lane * pitch * 4),
+                              S + ((int64_t)s * nsdm + g) * s_stride + a0, bytes, full(slot));
+            issued++;
+            if (++slot == stages) {
+                slot = 0;
+                par ^= 1u;
             }
         }
-        __syncthreads();
+        for (int st = max(0, issued - stages); st < issued; st++)
+            ok = __all_sync(0xffffffffu, ptx::mbar_wait(full(st % stages), (uint32_t)(st / stages) & 1u,
+                                                        2 * kS2Budget)) && ok;
+        if (!ok && lane == 0) atomicExch(err, 1);
+        return;
+    }
+    const int d0 = g * group, gcount = min(group, ndm - d0);
+    const int n = warp + kS2Warps < gcount ? 2 : (warp < gcount ? 1 : 0);  // trials of this warp
+    uint32_t acc[2][32];
 #pragma unroll
-        for (int i = 0; i < kMaxGroup; i++) {
-            if (i < gcount) {
-                for (int r = 0; r < sc; r++) {
-                    const int32_t *row = rows + r * row_len + soff[i * nsub + s0 + r] + threadIdx.x;
+    for (int i = 0; i < 2; i++)
 #pragma unroll
-                    for (int j = 0; j < 4; j++) acc[i][j] += row[kS2Threads * j];
+        for (int k = 0; k < 32; k++) acc[i][k] = 0;
+    // lane i * rows + r holds the offset of trial i in row r of the stage (loaded a stage ahead)
+    const int li = lane / rows, lr = lane - li * rows;
+    const int32_t *orow = off2 + (int64_t)(d0 + min(warp + kS2Warps * min(li, 1), gcount - 1)) * nsub;
+    auto offset = [&](int st) {
+        const int s = st * rows + lr;
+        return li < 2 && s < nsub ? __ldg(orow + s) : 0;
+    };
+    int nxt = offset(0), slot = 0;
+    uint32_t par = 0;
+    for (int st = 0; st < nst; st++) {
+        const int cur = nxt;
+        if (st + 1 < nst) nxt = offset(st + 1);
+        if (!__all_sync(0xffffffffu, ptx::mbar_wait(full(slot), par, kS2Budget))) {
+            if (lane == 0) atomicExch(err, 1);
+            return;
+        }
+        const uint32_t base = sm0 + (uint32_t)slot * stage_bytes + 4u * (uint32_t)lane;
+        const int rc = min(rows, nsub - st * rows);
+#pragma unroll
+        for (int i = 0; i < 2; i++) {
+            if (i < n) {
+                int r = 0;
+                for (; r + 2 <= rc; r += 2) {
+                    const uint32_t p = base + 4u * (uint32_t)(r * pitch + __shfl_sync(0xffffffffu, cur, i * rows + r));
+                    const uint32_t q = base + 4u * (uint32_t)((r + 1) * pitch + __shfl_sync(0xffffffffu, cur, i * rows + r + 1));
+#pragma unroll
+                    for (int h = 0; h < 32; h += 8) {
+                        uint32_t x[8], y[8];
+                        ptx::lds_words<8>(p + 128u * (uint32_t)h, x);
+                        ptx::lds_words<8>(q + 128u * (uint32_t)h, y);
+#pragma unroll
+                        for (int k = 0; k < 8; k++) acc[i][h + k] += x[k] + y[k];
+                    }
+                }
+                if (r < rc) {
+                    const uint32_t p = base + 4u * (uint32_t)(r * pitch + __shfl_sync(0xffffffffu, cur, i * rows + r));
+#pragma unroll
+                    for (int h = 0; h < 32; h += 8) {
+                        uint32_t x[8];
+                        ptx::lds_words<8>(p + 128u * (uint32_t)h, x);
+#pragma unroll
+                        for (int k = 0; k < 8; k++) acc[i][h + k] += x[k];
+                    }
                 }
             }
         }
+        __syncwarp();
+        if (lane == 0) ptx::mbar_arrive(empty(slot));
+        if (++slot == stages) {
+            slot = 0;
+            par ^= 1u;
+        }
     }
 #pragma unroll
-    for (int i = 0; i < kMaxGroup; i++) {
-        if (i < gcount) {
-            int32_t *o = D + (int64_t)(d0 + i) * d_stride;
+    for (int i = 0; i < 2; i++) {
+        if (i < n) {
+            int32_t *o = D + (int64_t)(d0 + warp + kS2Warps * i) * d_stride + t0 + lane;
+            const int64_t left = n_out - t0 - lane;
 #pragma unroll
-            for (int j = 0; j < 4; j++) {
-                const int64_t t = t0 + threadIdx.x + kS2Threads * j;
-                if (t < n_out) o[t] = acc[i][j];
-            }
+            for (int k = 0; k < 32; k++)
+                if (32 * k < left) __stcs(o + 32 * k, (int32_t)acc[i][k]);
         }
     }
 }
@@ -210,7 +299,7 @@ struct gsp_subband_s {
     int32_t *d_min2 = nullptr;       // [nsdm][nsub]
     int32_t *d_off2 = nullptr;       // [ndm][nsub]
     int *d_err = nullptr;
-    int row_len = 0, chunk = 0, smem = 0;
+    int pitch = 0, rows = 0, stages = 0, smem = 0;  // shared-memory ring of stage 2
     int num_sms = 0;
     int32_t launches = 0;
 };
@@ -354,15 +443,27 @@ gsp_status gsp_subband_create(gsp_subband_t *out, const gsp_plan_desc *desc, int
             b->off2[(size_t)d * nsub + s] = o;
             spread = std::max<int64_t>(spread, o);
         }
-    b->row_len = (int)(((int64_t)kS2Tile + spread + 3) & ~(int64_t)3);
-    const int64_t fixed = (int64_t)kMaxGroup * nsub * 4;
-    const int64_t budget = 100 * 1024 - fixed;
-    b->chunk = (int)std::max<int64_t>(1, std::min<int64_t>(nsub, budget / ((int64_t)b->row_len * 4)));
-    b->smem = (int)(fixed + (int64_t)b->chunk * b->row_len * 4);
-    if (spread > (1 << 20) || b->smem > 227 * 1024) {
+    // a row's window: the tile, the spread of the offsets and the 3 samples down to the
+    // 16-byte boundary; the ring takes half an SM's shared memory (two CTAs) where it can
+    const int64_t pitch = ((int64_t)kS2Tile + spread + 3 + 3) & ~(int64_t)3;
+    auto fit = [&](int64_t budget, int rows) {
+        return (int)std::min<int64_t>(8, budget / (pitch * 4 * rows + 16));
+    };
+    b->pitch = (int)pitch;
+    b->rows = std::min(kS2Rows, nsub);
+    b->stages = fit(112 * 1024, b->rows);
+    while (b->stages < 3 && b->rows > 1) {
+        b->rows /= 2;
+        b->stages = fit(112 * 1024, b->rows);
+    }
+    if (b->stages < 2) b->stages = fit(227 * 1024, b->rows);
+    // plans are accepted while a row and 64 bytes per sub-band fit an SM's shared memory
+    if (spread > (1 << 20) || b->stages < 1 ||
+        (int64_t)kMaxGroup * nsub * 4 + (((kS2Tile + spread + 3) & ~(int64_t)3) * 4) > 227 * 1024) {
         free_subband(b);
         return GSP_ERR_INVALID_ARG;
     }
+    b->smem = (int)(b->stages * (b->rows * pitch * 4 + 16));
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&b->num_sms, cudaDevAttrMultiProcessorCount, dev);
@@ -402,8 +503,12 @@ gsp_status gsp_subband_create(gsp_subband_t *out, const gsp_plan_desc *desc, int
         return st;
     }
     e = cudaMemcpy(b->d_min2, b->min2.data(), b->min2.size() * 4, cudaMemcpyHostToDevice);
-    if (e == cudaSuccess)
-        e = cudaMemcpy(b->d_off2, b->off2.data(), b->off2.size() * 4, cudaMemcpyHostToDevice);
+    // on the device the offsets count from the 16-byte boundary below a row's start
+    std::vector<int32_t> off(b->off2);
+    for (int d = 0; d < ndm; d++)
+        for (int s = 0; s < nsub; s++)
+            off[(size_t)d * nsub + s] += b->min2[(size_t)(d / group) * nsub + s] & 3;
+    if (e == cudaSuccess) e = cudaMemcpy(b->d_off2, off.data(), off.size() * 4, cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemset(b->d_err, 0, sizeof(int));
     if (e == cudaSuccess && b->smem > 48 * 1024)
         e = cudaFuncSetAttribute(subband_sum_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -481,9 +586,9 @@ gsp_status gsp_subband_dedisperse(gsp_subband_t b, const uint8_t *d_x, int64_t n
     }
     // stage 2: sums of the sub-band series, shifted by the reference delays
     dim3 grid((unsigned)((n_out + kS2Tile - 1) / kS2Tile), (unsigned)b->nsdm);
-    subband_sum_kernel<<<grid, kS2Threads, b->smem, s>>>(
-        b->d_S, b->s_stride, b->nsdm, b->nsub, n1, b->d_min2, b->d_off2, b->ndm, b->group,
-        b->row_len, b->chunk, n_out, d_out, out_stride);
+    subband_sum_kernel<<<grid, (kS2Warps + 1) * 32, b->smem, s>>>(
+        b->d_S, b->s_stride, b->nsdm, b->nsub, b->d_min2, b->d_off2, b->ndm, b->group, b->pitch,
+        b->rows, b->stages, n_out, d_out, out_stride, b->d_err);
     b->launches += 1;
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) {
