@@ -659,33 +659,46 @@ bool mma_plan_tables(const int32_t *delays, int ndm, int C, bool rev, MmaTables 
     t->frames.clear();
     t->rmax = 0;
     t->mean_cols_r = 0.0;
+    // a block's delays by position, the 16 trials side by side (loops over them vectorise)
+    std::vector<int32_t> dl((size_t)C * kKdm);
+    struct Range {
+        int lo, hi;
+    };
+    auto range_of = [](const int32_t *x, const int32_t *y) {  // of x[i] - y[i] over the block
+        int32_t lo = INT32_MAX, hi = INT32_MIN;
+        for (int i = 0; i < kKdm; i++) {
+            const int32_t v = x[i] - y[i];
+            lo = std::min(lo, v);
+            hi = std::max(hi, v);
+        }
+        return Range{lo, hi};
+    };
     for (int b = 0; b < nblk; b++) {
-        const int32_t *row[kKdm];
-        for (int i = 0; i < kKdm; i++) row[i] = delays + (size_t)std::min(ndm - 1, b * kKdm + i) * C;
-        auto at = [&](int i, int pos) { return row[i][rev ? C - 1 - pos : pos]; };
-        int R[kKdm] = {}, ref[kKdm];
+        for (int i = 0; i < kKdm; i++) {
+            const int32_t *row = delays + (size_t)std::min(ndm - 1, b * kKdm + i) * C;
+            int32_t *d = dl.data() + i;
+            if (rev)
+                for (int pos = 0; pos < C; pos++) d[(size_t)pos * kKdm] = row[C - 1 - pos];
+            else
+                for (int pos = 0; pos < C; pos++) d[(size_t)pos * kKdm] = row[pos];
+        }
+        int32_t R[kKdm] = {};
         bool first = true;
         int rmax = 0;
         for (int p0 = 0; p0 < C;) {
             // centre the frame on the furthest channel whose delays differ from those of
             // p0 by amounts within 8 samples of each other, with moves of at most 16
+            const int32_t *d0 = dl.data() + (size_t)p0 * kKdm;
             int best = p0;
             for (int pos = p0; pos < C; pos++) {
-                int lo = INT32_MAX, hi = INT32_MIN, elo = INT32_MAX, ehi = INT32_MIN;
-                for (int i = 0; i < kKdm; i++) {
-                    const int v = at(i, pos), dv = v - at(i, p0), ev = v - R[i];
-                    lo = std::min(lo, dv);
-                    hi = std::max(hi, dv);
-                    elo = std::min(elo, ev);
-                    ehi = std::max(ehi, ev);
-                }
-                if (hi - lo > kMaxShift || (!first && ehi - elo > kMaxMove)) break;
+                const int32_t *d = dl.data() + (size_t)pos * kKdm;
+                const Range dv = range_of(d, d0), ev = range_of(d, R);
+                if (dv.hi - dv.lo > kMaxShift || (!first && ev.hi - ev.lo > kMaxMove)) break;
                 best = pos;
             }
-            for (int i = 0; i < kKdm; i++) ref[i] = at(i, best);
+            const int32_t *ref = dl.data() + (size_t)best * kKdm;
             for (bool more = true; more;) {
-                int elo = INT32_MAX;
-                for (int i = 0; i < kKdm; i++) elo = std::min(elo, ref[i] - R[i]);
+                const int elo = range_of(ref, R).lo;
                 MmaFrame fr;
                 fr.pos = p0;
                 more = false;
@@ -698,7 +711,7 @@ bool mma_plan_tables(const int32_t *delays, int ndm, int C, bool rev, MmaTables 
                     }
                     fr.e[i] = first ? 0 : (uint8_t)e;
                     R[i] += e;
-                    rmax = std::max(rmax, R[i]);
+                    rmax = std::max(rmax, (int)R[i]);
                 }
                 fr.rmax = rmax;
                 if (rmax > 8 * kCols) return false;
@@ -707,16 +720,12 @@ bool mma_plan_tables(const int32_t *delays, int ndm, int C, bool rev, MmaTables 
             }
             int pos = p0;
             for (; pos < C; pos++) {
-                int lo = INT32_MAX, hi = INT32_MIN;
-                for (int i = 0; i < kKdm; i++) {
-                    const int v = at(i, pos) - R[i];
-                    lo = std::min(lo, v);
-                    hi = std::max(hi, v);
-                }
-                if (hi - lo > kMaxShift) break;
-                t->base[(size_t)b * C + pos] = lo;
+                const int32_t *d = dl.data() + (size_t)pos * kKdm;
+                const Range v = range_of(d, R);
+                if (v.hi - v.lo > kMaxShift) break;
+                t->base[(size_t)b * C + pos] = v.lo;
                 uint8_t *s = t->shift.data() + ((size_t)b * nchunk + pos / kChunk) * kKdm * kChunk + pos % kChunk;
-                for (int i = 0; i < kKdm; i++) s[i * kChunk] = (uint8_t)(at(i, pos) - R[i] - lo);
+                for (int i = 0; i < kKdm; i++) s[i * kChunk] = (uint8_t)(d[i] - R[i] - v.lo);
                 int32_t &cr = t->crmax[(size_t)b * nchunk + pos / kChunk];
                 cr = std::max(cr, rmax);
                 t->mean_cols_r += rmax;

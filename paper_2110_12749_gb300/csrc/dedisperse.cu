@@ -986,17 +986,21 @@ bool plan_dedisperse_tiled(gsp_plan_s *p, TiledTables *tab) {
         std::vector<int32_t> &bm = tab->blkmin[o];
         bm.assign((size_t)nblk * C, 0);
         std::vector<int64_t> chspread((size_t)C, 0);  // per channel, over all blocks
+        // row by row (the delay table is walked in storage order, and the loops vectorise)
+        std::vector<int32_t> hi((size_t)C);
         for (int b = 0; b < nblk; b++) {
-            for (int c = 0; c < C; c++) {
-                int32_t lo = INT32_MAX, hi = 0;
-                for (int d = b * kdm; d < std::min(ndm, (b + 1) * kdm); d++) {
-                    const int32_t v = p->delays_h[(size_t)d * C + c];
-                    lo = std::min(lo, v);
-                    hi = std::max(hi, v);
+            int32_t *lo = bm.data() + (size_t)b * C;
+            const int32_t *first = p->delays_h.data() + (size_t)b * kdm * C;
+            std::copy(first, first + C, lo);
+            std::copy(first, first + C, hi.begin());
+            for (int d = b * kdm + 1; d < std::min(ndm, (b + 1) * kdm); d++) {
+                const int32_t *v = p->delays_h.data() + (size_t)d * C;
+                for (int c = 0; c < C; c++) {
+                    lo[c] = std::min(lo[c], v[c]);
+                    hi[c] = std::max(hi[c], v[c]);
                 }
-                bm[(size_t)b * C + c] = lo;
-                chspread[c] = std::max<int64_t>(chspread[c], (int64_t)hi - lo);
             }
+            for (int c = 0; c < C; c++) chspread[c] = std::max<int64_t>(chspread[c], (int64_t)hi[c] - lo[c]);
         }
         int64_t spread = 0;
         for (int c = 0; c < C; c++) spread = std::max(spread, chspread[c]);

@@ -50,12 +50,17 @@ gsp_status compute_delays(const gsp_plan_desc *d, const std::vector<double> &dms
     const double ftop = d->f_lo_mhz + ((double)(C - 1) + 0.5) * df;
     const double inv_top2 = 1.0 / (ftop * ftop);
     double margin = 1.0;
+    // 1/f_c^2 - 1/f_top^2 of every channel, once (the same values in the same operation order)
+    std::vector<double> law((size_t)C);
+    for (int64_t c = 0; c < C; c++) {
+        const int64_t k = d->freq_descending ? (C - 1 - c) : c;
+        const double f = d->f_lo_mhz + ((double)k + 0.5) * df;
+        law[c] = 1.0 / (f * f) - inv_top2;
+    }
     for (size_t i = 0; i < dms.size(); i++) {
         const double dm = dms[i];
         for (int64_t c = 0; c < C; c++) {
-            const int64_t k = d->freq_descending ? (C - 1 - c) : c;
-            const double f = d->f_lo_mhz + ((double)k + 0.5) * df;
-            const double x = 4.148808e3 * dm * (1.0 / (f * f) - inv_top2) / d->t_samp_s;
+            const double x = 4.148808e3 * dm * law[c] / d->t_samp_s;
             const double fl = std::floor(x);
             const double m = std::fabs((x - fl) - 0.5);
             if (m < margin) margin = m;
