@@ -5,18 +5,19 @@
 //
 // Network: three conv 3x3 (pad 1) + bias + ReLU + 2x2 max-pool layers
 // (1 -> 8 -> 16 -> 32 channels, 64x64 -> 8x8), fc 2048 -> 96 + ReLU, fc 96 -> 2.
-// Activations are NHWC.  Every convolution of a training pass is an im2col
-// GEMM on the tcgen05 tensor cores (tc_gemm.cu), BF16 operands and FP32
-// accumulation in tensor memory, bias and ReLU fused into the epilogue.  An
-// inference pass fuses each conv layer with its bias, ReLU and pool at the
-// same rounding points: layer 0 (one input channel, K = 9) on the CUDA cores,
-// layers 1 and 2 as implicit GEMMs on the tensor cores that gather their taps
-// straight from the activations.  fc 2048 -> 96 and the
-// back-propagated products of both fc layers and the convolutions are GEMMs
-// too (weight gradients with split-K over the batch pixels).  The 96 -> 2
-// layer, the loss, pooling, im2col / col2im, bias gradients and Adam are
-// elementwise kernels in FP32.  Every operand of a product is rounded to
-// bf16 (nearest even), at the same points as the CPU oracle.
+// Activations are NHWC.  Each conv layer is one kernel with its bias, ReLU and
+// pool: layer 0 (one input channel, K = 9) on the CUDA cores, layers 1 and 2 as
+// implicit GEMMs on the tcgen05 tensor cores (BF16 operands, FP32 accumulation in
+// tensor memory) that gather their taps straight from the activations; the same
+// kernels run a training pass and then also keep the ReLU outputs and the pool's
+// argmaxes.  Back-propagation: input gradients of layers 1 and 2 by the same implicit
+// GEMM with mirrored taps; conv weight gradients on the CUDA cores from the pooled
+// gradients (one nonzero per pooling window); both products of fc 2048 -> 96 by the
+// tcgen05 GEMM (tc_gemm.cu).  The 96 -> 2 layer, the loss, the pool's way back,
+// bias gradients and Adam are elementwise kernels in FP32.  Every operand of a
+// product is rounded to bf16 (nearest even), at the same points as the CPU oracle.
+// A training step at 256 snippets takes 230 us (im2col matrices, their transposes
+// and GEMMs for every product: 860 us).
 #include <algorithm>
 #include <cmath>
 #include <cstring>
@@ -45,6 +46,7 @@ __host__ __device__ constexpr int side_of(int l) { return l == 0 ? 64 : (l == 1 
 __host__ __device__ constexpr int round8(int v) { return (v + 7) & ~7; }
 __host__ __device__ constexpr int kdim(int l) { return 9 * cin_of(l); }         // im2col K
 __host__ __device__ constexpr int kpad(int l) { return round8(kdim(l)); }
+constexpr int kGradRows = 16;  // rows of the input-gradient weights (at least Cin of layers 1, 2)
 
 // Parameter offsets in the flat FP32 vector (order w1 b1 w2 b2 w3 b3 w4 b4 w5 b5,
 // each in the oracle's layout: conv w[co][ci][ky][kx], fc w[out][in]).
@@ -68,49 +70,6 @@ Offsets offsets() {
 
 // ------------------------------------------------------------- elementwise
 
-// im2col of an NHWC activation (layer 0: the FP32 snippets, rounded to bf16
-// here): col[(b, y, x)][(ky * 3 + kx) * CIN + ci] = a[b][y + ky - 1][x + kx - 1][ci],
-// zero outside the image and in the padding columns K..Kp.  One thread per
-// pixel writes its whole row of Kp values in 16-byte pieces (consecutive
-// threads write consecutive rows); channel taps are read 16 bytes at a time
-// when CIN is a multiple of 8.
-template <typename T, int CIN>
-__global__ void __launch_bounds__(256) im2col_kernel(const T *__restrict__ a, int B, int H,
-                                                     bf16 *__restrict__ col) {
-    constexpr int K = 9 * CIN, KP = (K + 7) & ~7;
-    const int64_t npix = (int64_t)B * H * H;
-    for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < npix;
-         p += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t b = p / (H * H);
-        const int rem = (int)(p - b * H * H);
-        const int y = rem / H, x = rem - (rem / H) * H;
-        __align__(16) bf16 row[KP];
-#pragma unroll
-        for (int tap = 0; tap < 9; tap++) {
-            const int yy = y + tap / 3 - 1, xx = x + tap % 3 - 1;
-            const bool in = yy >= 0 && yy < H && xx >= 0 && xx < H;
-            const T *src = a + ((b * H + yy) * H + xx) * CIN;
-            if constexpr (CIN % 8 == 0 && sizeof(T) == 2) {
-#pragma unroll
-                for (int c8 = 0; c8 < CIN / 8; c8++) {
-                    uint4 v = make_uint4(0u, 0u, 0u, 0u);
-                    if (in) v = __ldg(reinterpret_cast<const uint4 *>(src) + c8);
-                    *reinterpret_cast<uint4 *>(&row[tap * CIN + c8 * 8]) = v;
-                }
-            } else {
-#pragma unroll
-                for (int ci = 0; ci < CIN; ci++)
-                    row[tap * CIN + ci] = __float2bfloat16_rn(in ? (float)src[ci] : 0.0f);
-            }
-        }
-#pragma unroll
-        for (int k = K; k < KP; k++) row[k] = __float2bfloat16_rn(0.0f);
-        uint4 *dst = reinterpret_cast<uint4 *>(col + p * KP);
-#pragma unroll
-        for (int q = 0; q < KP / 8; q++) dst[q] = *reinterpret_cast<const uint4 *>(&row[q * 8]);
-    }
-}
-
 // fma(a, b.x, c.x), fma(a, b.y, c.y) as one packed instruction (two IEEE
 // single-precision FMAs, the same results as two fmaf): half the issue slots
 __device__ __forceinline__ float2 fma_pair(float a, float2 b, float2 c) {
@@ -124,16 +83,16 @@ __device__ __forceinline__ float2 fma_pair(float a, float2 b, float2 c) {
     return r;
 }
 
-// Layer 0 of an inference pass: conv 3x3 (1 -> 8, pad 1) + bias + ReLU + 2x2
-// max-pool straight from the FP32 snippets, on the CUDA cores: with one input
-// channel the product has K = 9, too short for the tensor pipe to pay for its
-// staging.  The rounding points are those of the im2col + GEMM + pool path:
-// inputs and weights in bf16, the nine products and the bias summed in FP32
-// (in the same order), the pooled maximum rounded to bf16.  One thread per pair
-// of horizontally adjacent pooled pixels reads its 4 x 6 input patch; per
-// channel it loads the nine weights once and computes the pair's 2 x 4 conv
-// outputs, then writes the two pixels' 8 bf16 results as two 16-byte stores
-// (NHWC, as pool_kernel<8>).  Channels 2p and 2p + 1 share each packed FMA.
+// Layer 0: conv 3x3 (1 -> 8, pad 1) + bias + ReLU + 2x2 max-pool straight from
+// the FP32 snippets, on the CUDA cores: with one input channel the product has
+// K = 9, too short for the tensor pipe to pay for its staging.  Rounding points:
+// inputs and weights in bf16, the nine products and the bias summed in FP32, the
+// pooled maximum rounded to bf16.  One thread per pair of horizontally adjacent
+// pooled pixels reads its 4 x 6 input patch; per channel pair it loads the nine
+// weights once and computes the 2 x 4 conv outputs (channels 2p and 2p + 1 share
+// each packed FMA), then writes the two pixels' 8 bf16 results as two 16-byte
+// stores (NHWC).  For inference; a training pass, which keeps the pre-pool values, runs
+// conv0_train_tc_kernel.
 __global__ void __launch_bounds__(256) conv0_pool_kernel(const float *__restrict__ x, int B,
                                                          const bf16 *__restrict__ W0,
                                                          const float *__restrict__ b0,
@@ -203,101 +162,161 @@ __global__ void __launch_bounds__(256) conv0_pool_kernel(const float *__restrict
     }
 }
 
-// 2x2 max-pool of the ReLU'd pre-activations z (FP32 NHWC [B][H][H][C]):
-// out bf16 [B][H/2][H/2][C], idx = argmax in (0,0), (0,1), (1,0), (1,1) order
-// (first maximum wins).  One thread per pooled pixel, all C channels (float4
-// loads).
-template <int C>
-__global__ void __launch_bounds__(256) pool_kernel(const float *__restrict__ z, int B, int H,
-                                                   bf16 *__restrict__ out,
-                                                   uint8_t *__restrict__ idx) {
-    const int H2 = H / 2;
-    const int64_t total = (int64_t)B * H2 * H2;
-    for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < total;
-         q += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t b = q / (H2 * H2);
-        const int rem = (int)(q - b * H2 * H2);
-        const int y = rem / H2, x = rem - (rem / H2) * H2;
-        const float *p0 = z + ((b * H + 2 * y) * H + 2 * x) * C;
-        const float *src[4] = {p0, p0 + C, p0 + (int64_t)H * C, p0 + (int64_t)H * C + C};
-#pragma unroll
-        for (int c4 = 0; c4 < C / 4; c4++) {
-            float4 v[4];
-#pragma unroll
-            for (int k = 0; k < 4; k++) v[k] = __ldg(reinterpret_cast<const float4 *>(src[k]) + c4);
-            float m[4] = {v[0].x, v[0].y, v[0].z, v[0].w};
-            uint32_t kk[4] = {0, 0, 0, 0};
-#pragma unroll
-            for (int k = 1; k < 4; k++) {
-                const float w[4] = {v[k].x, v[k].y, v[k].z, v[k].w};
-#pragma unroll
-                for (int e = 0; e < 4; e++)
-                    if (w[e] > m[e]) {
-                        m[e] = w[e];
-                        kk[e] = (uint32_t)k;
-                    }
-            }
-            const int64_t o = q * C + c4 * 4;
-#pragma unroll
-            for (int e = 0; e < 4; e++) out[o + e] = __float2bfloat16_rn(m[e]);
-            *reinterpret_cast<uint32_t *>(idx + o) = kk[0] | (kk[1] << 8) | (kk[2] << 16) | (kk[3] << 24);
-        }
-    }
-}
-
 // Back through the pool and the ReLU: g[b][y][x][c] = ga[b][y/2][x/2][c] if (y, x)
-// is the window's argmax and z > 0, else 0.  Writes bf16 g as [P][C] and as
-// its transpose [C][P] (P = B*H*H pixels, ldT >= P), and adds FP32 per-channel
-// sums into db.
-__global__ void pool_back_kernel(const float *__restrict__ ga, const uint8_t *__restrict__ idx,
-                                 const float *__restrict__ z, int B, int H, int C,
-                                 bf16 *__restrict__ g, bf16 *__restrict__ gT, int64_t ldT,
-                                 float *__restrict__ db) {
-    extern __shared__ float sdb[];
+// is the window's argmax and its pooled value a > 0, else 0, as bf16 [P][C]
+// (P = B*H*H pixels); adds FP32 per-channel sums into db.  One thread per pooled
+// pixel and 8 channels: it reads the gradient, argmax and pooled value once
+// and writes the window's four pixels, 16 bytes each.  (A thread per pre-pool
+// element that also scattered a transpose took 65 us per layer at 256 snippets.)
+template <int C>
+__global__ void __launch_bounds__(256) pool_back_kernel(const float *__restrict__ ga,
+                                                        const uint8_t *__restrict__ idx,
+                                                        const bf16 *__restrict__ a, int B, int H,
+                                                        bf16 *__restrict__ g, float *__restrict__ db) {
+    constexpr int G = C / 8;  // channel groups; 256 and the grid's stride are multiples of it
+    __shared__ float sdb[C];
     for (int c = threadIdx.x; c < C; c += blockDim.x) sdb[c] = 0.0f;
     __syncthreads();
     const int H2 = H / 2;
-    const int64_t P = (int64_t)B * H * H;
-    const int64_t total = P * C;
+    const int64_t total = (int64_t)B * H2 * H2 * G;
+    float sum[8];
+#pragma unroll
+    for (int e = 0; e < 8; e++) sum[e] = 0.0f;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total;
          i += (int64_t)gridDim.x * blockDim.x) {
-        const int c = (int)(i % C);
-        const int64_t p = i / C;
-        const int x = (int)(p % H), y = (int)((p / H) % H);
-        const int64_t b = p / ((int64_t)H * H);
-        const int64_t q = ((b * H2 + y / 2) * H2 + x / 2) * C + c;
-        const int k = (y & 1) * 2 + (x & 1);
-        float v = 0.0f;
-        if (idx[q] == k && z[i] > 0.0f) v = ga[q];
-        g[i] = __float2bfloat16_rn(v);
-        gT[(int64_t)c * ldT + p] = __float2bfloat16_rn(v);
-        if (v != 0.0f) atomicAdd(&sdb[c], v);
+        const int64_t q = i / G;
+        const int c8 = (int)(i - q * G);
+        const int64_t b = q / (H2 * H2);
+        const int rem = (int)(q - b * H2 * H2);
+        const int y2 = rem / H2, x2 = rem - (rem / H2) * H2;
+        const float4 f0 = __ldg(reinterpret_cast<const float4 *>(ga + q * C) + 2 * c8);
+        const float4 f1 = __ldg(reinterpret_cast<const float4 *>(ga + q * C) + 2 * c8 + 1);
+        const uint2 k = __ldg(reinterpret_cast<const uint2 *>(idx + q * C) + c8);
+        const uint4 av = __ldg(reinterpret_cast<const uint4 *>(a + q * C) + c8);
+        const float f[8] = {f0.x, f0.y, f0.z, f0.w, f1.x, f1.y, f1.z, f1.w};
+        const uint32_t ab[4] = {av.x, av.y, av.z, av.w};
+        __align__(16) bf16 o[4][8];
+#pragma unroll
+        for (int e = 0; e < 8; e++) {
+            // pooled values are >= 0: positive when any of their bits are set
+            const bool pos = ((ab[e >> 1] >> (16 * (e & 1))) & 0x7fffu) != 0u;
+            const float v = pos ? f[e] : 0.0f;
+            const uint32_t at = ((e < 4 ? k.x : k.y) >> (8 * (e & 3))) & 0xffu;
+            sum[e] += v;
+            const bf16 w = __float2bfloat16_rn(v), zero = __float2bfloat16_rn(0.0f);
+#pragma unroll
+            for (int p = 0; p < 4; p++) o[p][e] = at == (uint32_t)p ? w : zero;
+        }
+#pragma unroll
+        for (int p = 0; p < 4; p++)
+            *reinterpret_cast<uint4 *>(g + ((b * H + 2 * y2 + p / 2) * H + 2 * x2 + p % 2) * C + 8 * c8) =
+                *reinterpret_cast<const uint4 *>(o[p]);
+    }
+#pragma unroll
+    for (int e = 0; e < 8; e++) {
+        // lanes of the same channel group are G apart
+        for (int o = 16; o >= G; o >>= 1) sum[e] += __shfl_xor_sync(0xffffffffu, sum[e], o);
+        if ((threadIdx.x & 31) < G) atomicAdd(&sdb[8 * (threadIdx.x & (G - 1)) + e], sum[e]);
     }
     __syncthreads();
     for (int c = threadIdx.x; c < C; c += blockDim.x)
         if (sdb[c] != 0.0f) atomicAdd(&db[c], sdb[c]);
 }
 
-// col2im (gather form): ga[b][y][x][ci] = sum over taps (ky, kx) of
-// dcol[(b, y - ky + 1, x - kx + 1)][(ky * 3 + kx) * Cin + ci].
-__global__ void col2im_kernel(const float *__restrict__ dcol, int B, int H, int Cin, int Kp,
-                              float *__restrict__ ga) {
-    const int64_t total = (int64_t)B * H * H * Cin;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        const int ci = (int)(i % Cin);
-        const int64_t p = i / Cin;
-        const int x = (int)(p % H), y = (int)((p / H) % H);
-        const int64_t b = p / ((int64_t)H * H);
-        float s = 0.0f;
+// Weight gradient of a conv layer, dw[co][ci][ky][kx] += sum over the pixels of
+// gz[p][co] * act[p + (ky - 1, kx - 1)][ci], from the pooled gradient: a pooling
+// window has one nonzero gz per channel, at its argmax, so a quarter of the
+// products of the dense sum do.  A CTA stages a strip of its image's activation (bf16 with
+// a zero border; layer 0: the FP32 snippet rounded here) and its windows' bf16
+// gradients; a thread owns output channel co and CP input channels and
+// keeps their 9 CP sums in registers over all its windows.  Operands in bf16,
+// exact products, FP32 sums, added atomically at the end.  Bound by the shared loads
+// (one per tap and window).  Replaces an im2col, two transposes and a split-K
+// GEMM whose 128-row tiles held 8 to 32 rows of work.
+template <typename T, int CIN, int COUT, int SIDE>
+__global__ void __launch_bounds__(256) conv_dw_kernel(const T *__restrict__ act, int B,
+                                                      const float *__restrict__ ga,
+                                                      const uint8_t *__restrict__ idx,
+                                                      const bf16 *__restrict__ a,
+                                                      float *__restrict__ dw) {
+    constexpr int CP = CIN == 1 ? 1 : 2;               // input channels per thread
+    constexpr int kOwn = COUT * (CIN / CP);            // threads that cover the weights
+    constexpr int kSets = 256 / kOwn;                  // sets of them, sharing the windows
+    static_assert(256 % kOwn == 0, "whole sets");
+    constexpr int kStrips = SIDE / 16;                 // strips of 16 image rows per image
+    constexpr int kRows = 18, kPitch = SIDE + 2;       // a strip with its border
+    constexpr int PW = SIDE / 2, kWin = 8 * PW;        // pooling windows per strip
+    __shared__ __align__(16) bf16 sa[kRows * kPitch * CIN + 8];
+    __shared__ float sg[kWin * COUT];
+    const int tid = threadIdx.x, set = tid / kOwn, own = tid % kOwn;
+    const int co = own / (CIN / CP), cp = own % (CIN / CP);
+    float acc[9][CP];
 #pragma unroll
-        for (int tap = 0; tap < 9; tap++) {
-            const int yy = y - tap / 3 + 1, xx = x - tap % 3 + 1;
-            if (yy >= 0 && yy < H && xx >= 0 && xx < H)
-                s += dcol[((b * H + yy) * H + xx) * Kp + tap * Cin + ci];
+    for (int t = 0; t < 9; t++)
+#pragma unroll
+        for (int e = 0; e < CP; e++) acc[t][e] = 0.0f;
+    for (int64_t u = blockIdx.x; u < (int64_t)B * kStrips; u += gridDim.x) {
+        const int64_t b = u / kStrips;
+        const int y0 = (int)(u - b * kStrips) * 16;  // first image row of the strip
+        __syncthreads();
+        for (int i = tid; i < kRows * kPitch; i += 256) {
+            const int r = i / kPitch, c = i - r * kPitch;
+            const int yy = y0 + r - 1, xx = c - 1;
+            const bool in = yy >= 0 && yy < SIDE && xx >= 0 && xx < SIDE;
+            const T *src = act + ((b * SIDE + (in ? yy : 0)) * SIDE + (in ? xx : 0)) * CIN;
+            if constexpr (CIN % 8 == 0) {
+#pragma unroll
+                for (int c8 = 0; c8 < CIN / 8; c8++) {
+                    uint4 v = make_uint4(0u, 0u, 0u, 0u);
+                    if (in) v = __ldg(reinterpret_cast<const uint4 *>(src) + c8);
+                    *reinterpret_cast<uint4 *>(&sa[i * CIN + 8 * c8]) = v;
+                }
+            } else {
+                sa[i] = __float2bfloat16_rn(in ? (float)__ldg(src) : 0.0f);
+            }
         }
-        ga[i] = s;
+        // the windows' gradients, their argmax in the two lowest bits (the values are
+        // bf16: those bits are free in FP32)
+        const int64_t q0 = (b * PW + y0 / 2) * PW;
+        for (int i = tid; i < kWin * COUT; i += 256) {
+            const int64_t o = q0 * COUT + i;
+            const bool pos = __bfloat162float(a[o]) > 0.0f;
+            const float v = __bfloat162float(__float2bfloat16_rn(pos ? __ldg(ga + o) : 0.0f));
+            sg[i] = __uint_as_float(__float_as_uint(v) | (uint32_t)(idx[o] & 3u));
+        }
+        __syncthreads();
+        for (int w = set; w < kWin; w += kSets) {
+            const uint32_t bits = __float_as_uint(sg[w * COUT + co]);
+            if ((bits & 0x7ffffff0u) == 0u) continue;
+            const float gv = __uint_as_float(bits & ~3u);
+            const int wy = w / PW, wx = w % PW;
+            const int base = ((2 * wy + (int)((bits >> 1) & 1u)) * kPitch + 2 * wx + (int)(bits & 1u)) * CIN +
+                             cp * CP;
+#pragma unroll
+            for (int t = 0; t < 9; t++) {
+                const bf16 *p = &sa[base + ((t / 3) * kPitch + t % 3) * CIN];
+                if constexpr (CP == 2) {
+                    const uint32_t v = *reinterpret_cast<const uint32_t *>(p);
+                    acc[t][0] = fmaf(gv, __uint_as_float(v << 16), acc[t][0]);
+                    acc[t][CP - 1] = fmaf(gv, __uint_as_float(v & 0xffff0000u), acc[t][CP - 1]);
+                } else {
+                    acc[t][0] = fmaf(gv, __bfloat162float(*p), acc[t][0]);
+                }
+            }
+        }
     }
+    // the sets' sums, then one atomic per weight and CTA
+    __shared__ float red[COUT * CIN * 9];
+    for (int i = tid; i < COUT * CIN * 9; i += 256) red[i] = 0.0f;
+    __syncthreads();
+    {
+#pragma unroll
+        for (int t = 0; t < 9; t++)
+#pragma unroll
+            for (int e = 0; e < CP; e++) atomicAdd(&red[(co * CIN + cp * CP + e) * 9 + t], acc[t][e]);
+    }
+    __syncthreads();
+    for (int i = tid; i < COUT * CIN * 9; i += 256) atomicAdd(&dw[i], red[i]);
 }
 
 // bf16 transpose: out[c][r] = in[r][c] for r < R, c < Cc (32 x 32 tiles).
@@ -358,43 +377,41 @@ __global__ void loss_kernel(const float *__restrict__ z5, const int32_t *__restr
 }
 
 // Back through fc 96 -> 2 and the ReLU of fc1 (CUDA cores):
-//   dw5[o][k] = sum_b bf16(g5[b][o]) * a4[b][k],  db5[o] = sum_b g5[b][o]   (block 0)
+//   dw5[o][k] += sum_b bf16(g5[b][o]) * a4[b][k],  db5[o] += sum_b g5[b][o]
 //   g4[b][k]  = (sum_o bf16(g5[b][o]) * bf16(w5[o][k])) * [z4[b][k] > 0]
-// g4 is written as bf16 [B][96] and transposed [96][ldT]; db4 += FP32 sums.
+// g4 is written as bf16 [B][96] and transposed [96][ldT]; db4 += FP32 sums.  The
+// blocks take the snippets in turn and add their sums atomically (one block summing
+// dw5 over the whole batch took 39 us at 256 snippets).
 __global__ void fc2_back_kernel(const float *__restrict__ g5, const bf16 *__restrict__ a4,
                                 const float *__restrict__ w5, const float *__restrict__ z4,
                                 int B, float *__restrict__ dw5, float *__restrict__ db5,
                                 bf16 *__restrict__ g4, bf16 *__restrict__ g4T, int64_t ldT,
                                 float *__restrict__ db4) {
     const int k = threadIdx.x;  // kHid threads: one hidden unit each
-    if (blockIdx.x == 0) {
-        float s0 = 0.0f, s1 = 0.0f, t0 = 0.0f, t1 = 0.0f;
-        for (int b = 0; b < B; b++) {
-            const float a = (float)a4[b * kHid + k];
-            s0 = fmaf(__bfloat162float(__float2bfloat16_rn(g5[2 * b])), a, s0);
-            s1 = fmaf(__bfloat162float(__float2bfloat16_rn(g5[2 * b + 1])), a, s1);
-            t0 += g5[2 * b];
-            t1 += g5[2 * b + 1];
-        }
-        dw5[k] = s0;
-        dw5[kHid + k] = s1;
-        if (k == 0) {
-            db5[0] = t0;
-            db5[1] = t1;
-        }
-    }
     const float w0 = __bfloat162float(__float2bfloat16_rn(w5[k]));
     const float w1 = __bfloat162float(__float2bfloat16_rn(w5[kHid + k]));
-    float dsum = 0.0f;
+    float s0 = 0.0f, s1 = 0.0f, t0 = 0.0f, t1 = 0.0f, dsum = 0.0f;
     for (int b = blockIdx.x; b < B; b += gridDim.x) {
-        const float ga = __bfloat162float(__float2bfloat16_rn(g5[2 * b])) * w0 +
-                         __bfloat162float(__float2bfloat16_rn(g5[2 * b + 1])) * w1;
-        const float v = z4[b * kHid + k] > 0.0f ? ga : 0.0f;
+        const float2 g = __ldg(reinterpret_cast<const float2 *>(g5) + b);
+        const float h0 = __bfloat162float(__float2bfloat16_rn(g.x));
+        const float h1 = __bfloat162float(__float2bfloat16_rn(g.y));
+        const float act = (float)a4[b * kHid + k];
+        s0 = fmaf(h0, act, s0);
+        s1 = fmaf(h1, act, s1);
+        t0 += g.x;
+        t1 += g.y;
+        const float v = z4[b * kHid + k] > 0.0f ? h0 * w0 + h1 * w1 : 0.0f;
         g4[b * kHid + k] = __float2bfloat16_rn(v);
         g4T[(int64_t)k * ldT + b] = __float2bfloat16_rn(v);
         dsum += v;
     }
+    atomicAdd(&dw5[k], s0);
+    atomicAdd(&dw5[kHid + k], s1);
     atomicAdd(&db4[k], dsum);
+    if (k == 0) {
+        atomicAdd(&db5[0], t0);
+        atomicAdd(&db5[1], t1);
+    }
 }
 
 // Adam on the flat FP32 parameter vector (step number t >= 1).
@@ -412,14 +429,14 @@ __global__ void adam_kernel(float *__restrict__ p, const float *__restrict__ g,
     }
 }
 
-// bf16 GEMM copies of the conv weights: W[co][(ky*3+kx)*Cin + ci] (padded to
-// Kp) and its transpose WT[k][co] (ld Cout8), from w[co][ci][ky][kx]; and the
-// fc1 weight W4 [96][2048] with its transpose W4T [2048][96].
+// bf16 copies of the weights: conv W[co][(ky*3+kx)*Cin + ci] (padded to Kp) from
+// w[co][ci][ky][kx]; for the input gradients of layers 1 and 2 the product's other side,
+// WG[ci][(ky*3+kx)*Cout + co] (16 rows, zero past Cin); and the fc1 weight W4
+// [96][2048] with its transpose W4T [2048][96].
 __global__ void pack_kernel(const float *__restrict__ params, int64_t w1, int64_t w2, int64_t w3,
-                            int64_t w4, bf16 *__restrict__ W0, bf16 *__restrict__ W0T,
-                            bf16 *__restrict__ W1, bf16 *__restrict__ W1T, bf16 *__restrict__ W2,
-                            bf16 *__restrict__ W2T, bf16 *__restrict__ W4,
-                            bf16 *__restrict__ W4T) {
+                            int64_t w4, bf16 *__restrict__ W0, bf16 *__restrict__ W1,
+                            bf16 *__restrict__ W2, bf16 *__restrict__ WG1, bf16 *__restrict__ WG2,
+                            bf16 *__restrict__ W4, bf16 *__restrict__ W4T) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i < (int64_t)kHid * kFc) {
         const bf16 v = __float2bfloat16_rn(params[w4 + i]);
@@ -428,7 +445,7 @@ __global__ void pack_kernel(const float *__restrict__ params, int64_t w1, int64_
     }
     const int64_t woff[3] = {w1, w2, w3};
     bf16 *Wd[3] = {W0, W1, W2};
-    bf16 *WTd[3] = {W0T, W1T, W2T};
+    bf16 *WGd[3] = {nullptr, WG1, WG2};
 #pragma unroll
     for (int l = 0; l < kLayers; l++) {
         const int Cin = cin_of(l), Cout = cout_of(l), Kp = kpad(l);
@@ -439,21 +456,14 @@ __global__ void pack_kernel(const float *__restrict__ params, int64_t w1, int64_
                 const int tap = k / Cin, ci = k % Cin;
                 v = params[woff[l] + ((int64_t)co * Cin + ci) * 9 + tap];
             }
-            const bf16 b = __float2bfloat16_rn(v);
-            Wd[l][i] = b;
-            WTd[l][(int64_t)k * round8(Cout) + co] = b;
+            Wd[l][i] = __float2bfloat16_rn(v);
+        }
+        if (l > 0 && i < (int64_t)kGradRows * 9 * Cout) {
+            const int ci = (int)(i / (9 * Cout)), k = (int)(i % (9 * Cout));
+            const int tap = k / Cout, co = k % Cout;
+            WGd[l][i] = __float2bfloat16_rn(ci < Cin ? params[woff[l] + ((int64_t)co * Cin + ci) * 9 + tap] : 0.0f);
         }
     }
-}
-
-// Back to the oracle's conv weight-gradient layout: dw[co][ci][ky][kx] =
-// dW[co][(ky*3+kx)*Cin + ci].
-__global__ void unpack_conv_grad_kernel(const float *__restrict__ dW, int Cin, int Cout, int Kp,
-                                        float *__restrict__ dw) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= Cout * Cin * 9) return;
-    const int tap = i % 9, ci = (i / 9) % Cin, co = i / (9 * Cin);
-    dw[i] = dW[(int64_t)co * Kp + tap * Cin + ci];
 }
 
 }  // namespace
@@ -521,11 +531,29 @@ __device__ __forceinline__ void cp_async_wait() {
 //    and 2 through a 2 KB shared buffer.
 // Every wait is bounded; on a timeout the kernel sets *err, waits (bounded)
 // for its MMAs in flight and releases its tensor memory.
-template <int CIN, int COUT, int SIDE>
+//
+// kMode: kInfer as above; kTrain also stores the ReLU outputs z (FP32
+// [B][SIDE][SIDE][COUT]) and the pool's argmax idx (first maximum in (0,0),
+// (0,1), (1,0), (1,1) order); kGrad is the input gradient of such a layer: act
+// is the gradient of its pre-activations, the taps are mirrored, each tap's product
+// has its own accumulator (16 columns) and the nine are added in tap order, and the sums
+// are stored as FP32 z_out [B][SIDE][SIDE][nz] (nz <= 16 channels) without bias, ReLU
+// and pool.
+enum ConvMode { kInfer, kTrain, kGrad };
+
+// Tensor-memory columns of a CTA (a power of two, at least 32).
+__host__ __device__ constexpr uint32_t conv_tmem_cols(int cout, ConvMode mode) {
+    return mode == kGrad ? 256u : (cout < 32 ? 32u : (uint32_t)cout);
+}
+
+template <int CIN, int COUT, int SIDE, ConvMode kMode>
 __global__ void __launch_bounds__(128) conv_pool_solo_tc_kernel(const bf16 *__restrict__ act,
                                                                 int B, const bf16 *__restrict__ W,
                                                                 const float *__restrict__ bias,
-                                                                bf16 *__restrict__ out, int *err) {
+                                                                bf16 *__restrict__ out,
+                                                                float *__restrict__ z_out,
+                                                                uint8_t *__restrict__ idx, int nz,
+                                                                int *err) {
     constexpr int PW = SIDE / 2;
     static_assert(CIN % 8 == 0 && COUT % 16 == 0 && COUT <= 32, "shapes of layers 1 and 2");
     static_assert(SIDE == 16 || SIDE == 32, "16 x 16 or 32 x 32 images");
@@ -535,8 +563,10 @@ __global__ void __launch_bounds__(128) conv_pool_solo_tc_kernel(const bf16 *__re
     constexpr int KCS = NK16 * 2;
     constexpr uint32_t SBO = KCS * 128;
     constexpr int A_BYTES = 128 * KCS * 16;
-    constexpr uint32_t kCols = COUT < 32 ? 32u : (uint32_t)COUT;
+    constexpr uint32_t kCols = conv_tmem_cols(COUT, kMode);
     constexpr uint32_t kIdesc = tc::idesc_bf16(128, COUT);
+    constexpr int kTapSteps = kMode == kGrad ? CIN / 16 : NK16;  // K = 16 steps per accumulator
+    static_assert(kMode != kGrad || (COUT == 16 && CIN % 16 == 0), "one 16-column accumulator per tap");
     constexpr int KP = (K + 7) & ~7;
     extern __shared__ __align__(1024) uint8_t smem[];
     uint8_t *sA = smem, *sB = smem + A_BYTES;
@@ -544,13 +574,14 @@ __global__ void __launch_bounds__(128) conv_pool_solo_tc_kernel(const bf16 *__re
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(bar + 1);
     __shared__ float sbias[COUT];
     __shared__ __align__(16) float sx[SIDE == 32 ? 2 : 1][16][16];  // SIDE 32: odd rows' maxima
+    __shared__ uint32_t sk[SIDE == 32 ? 2 : 1][16];                 // and which column has them (training)
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int64_t ntiles = (int64_t)B * SIDE * SIDE / 128;
     const int64_t my = blockIdx.x < ntiles ? (ntiles - 1 - blockIdx.x) / gridDim.x + 1 : 0;
     if (warp == 0) tc::tmem_alloc(tc::smem_u32(tmem_slot), kCols);
     if (tid == 0) tc::mbar_init1(tc::smem_u32(bar));
-    for (int i = tid; i < COUT; i += 128) sbias[i] = bias[i];
+    for (int i = tid; i < COUT; i += 128) sbias[i] = kMode == kGrad ? 0.0f : bias[i];
     for (int idx = tid; idx < COUT * KCS; idx += 128) {
         const int n = idx % COUT, q = idx / COUT;
         uint4 v = make_uint4(0u, 0u, 0u, 0u);
@@ -578,7 +609,8 @@ __global__ void __launch_bounds__(128) conv_pool_solo_tc_kernel(const bf16 *__re
         const uint32_t dst = a_addr + (tid >> 3) * SBO + (tid & 7) * 16;
 #pragma unroll
         for (int tap = 0; tap < 9; tap++) {
-            const int dy = tap / 3 - 1, dx = tap % 3 - 1;
+            const int dy = kMode == kGrad ? 1 - tap / 3 : tap / 3 - 1;
+            const int dx = kMode == kGrad ? 1 - tap % 3 : tap % 3 - 1;
             const bool in = (unsigned)(y + dy) < (unsigned)SIDE && (unsigned)(x + dx) < (unsigned)SIDE;
             const bf16 *src = in ? base + (dy * SIDE + dx) * CIN : act;
 #pragma unroll
@@ -596,16 +628,49 @@ __global__ void __launch_bounds__(128) conv_pool_solo_tc_kernel(const bf16 *__re
         const int px = SIDE == 16 ? (lane & 15) >> 1 : lane >> 1;
         bf16 *dst = out + ((b * PW + py) * PW + px) * COUT;
         const bool writer = SIDE == 16 ? (lane & 17) == 0 : ((lane & 1) == 0 && (warp & 1) == 0);
+        if constexpr (kMode == kGrad) {
+            float v[16];
+            tc::tmem_ld16(taddr, v);
+#pragma unroll
+            for (int t = 1; t < 9; t++) {
+                float w[16];
+                tc::tmem_ld16(taddr + (uint32_t)(t * COUT), w);
+#pragma unroll
+                for (int c = 0; c < 16; c++) v[c] += w[c];
+            }
+            float4 *o = reinterpret_cast<float4 *>(z_out + (m0 + tid) * nz);
+#pragma unroll
+            for (int c = 0; c < 16; c += 4)
+                if (c < nz) o[c / 4] = make_float4(v[c], v[c + 1], v[c + 2], v[c + 3]);
+        } else {
 #pragma unroll
         for (int c0 = 0; c0 < COUT; c0 += 16) {
             float v[16];
             tc::tmem_ld16(taddr + (uint32_t)c0, v);
             float z[16];
+            uint32_t k1 = 0, k2 = 0;  // bit c: the window's maximum is in its second column / row
+#pragma unroll
+            for (int c = 0; c < 16; c++) z[c] = fmaxf(v[c] + sbias[c0 + c], 0.0f);
+            if constexpr (kMode == kTrain) {
+                float4 *o = reinterpret_cast<float4 *>(z_out + (m0 + tid) * COUT + c0);
+#pragma unroll
+                for (int c = 0; c < 16; c += 4) o[c / 4] = make_float4(z[c], z[c + 1], z[c + 2], z[c + 3]);
+            }
 #pragma unroll
             for (int c = 0; c < 16; c++) {
-                z[c] = fmaxf(v[c] + sbias[c0 + c], 0.0f);
-                z[c] = fmaxf(z[c], __shfl_xor_sync(0xffffffffu, z[c], 1));
-                if (SIDE == 16) z[c] = fmaxf(z[c], __shfl_xor_sync(0xffffffffu, z[c], 16));
+                const float r = __shfl_xor_sync(0xffffffffu, z[c], 1);
+                if (kMode == kTrain) k1 |= (r > z[c] ? 1u : 0u) << c;  // of even columns' lanes
+                z[c] = fmaxf(z[c], r);
+            }
+            if (SIDE == 16) {
+                const uint32_t kb = kMode == kTrain ? __shfl_xor_sync(0xffffffffu, k1, 16) : 0u;
+#pragma unroll
+                for (int c = 0; c < 16; c++) {
+                    const float r = __shfl_xor_sync(0xffffffffu, z[c], 16);
+                    if (kMode == kTrain) k2 |= (r > z[c] ? 1u : 0u) << c;
+                    z[c] = fmaxf(z[c], r);
+                }
+                k1 = (k1 & ~k2) | (kb & k2);
             }
             if (SIDE == 32) {
                 // the odd row of each row pair hands its column-pair maxima over
@@ -614,17 +679,23 @@ __global__ void __launch_bounds__(128) conv_pool_solo_tc_kernel(const bf16 *__re
                     for (int c = 0; c < 16; c += 4)
                         *reinterpret_cast<float4 *>(&sx[warp >> 1][lane >> 1][c]) =
                             make_float4(z[c], z[c + 1], z[c + 2], z[c + 3]);
+                    if (kMode == kTrain) sk[warp >> 1][lane >> 1] = k1;
                 }
                 __syncthreads();
                 if (writer) {
+                    const uint32_t kb = kMode == kTrain ? sk[warp >> 1][lane >> 1] : 0u;
 #pragma unroll
                     for (int c = 0; c < 16; c += 4) {
                         const float4 q = *reinterpret_cast<const float4 *>(&sx[warp >> 1][lane >> 1][c]);
+                        if (kMode == kTrain)
+                            k2 |= ((q.x > z[c] ? 1u : 0u) | (q.y > z[c + 1] ? 2u : 0u) |
+                                   (q.z > z[c + 2] ? 4u : 0u) | (q.w > z[c + 3] ? 8u : 0u)) << c;
                         z[c] = fmaxf(z[c], q.x);
                         z[c + 1] = fmaxf(z[c + 1], q.y);
                         z[c + 2] = fmaxf(z[c + 2], q.z);
                         z[c + 3] = fmaxf(z[c + 3], q.w);
                     }
+                    k1 = (k1 & ~k2) | (kb & k2);
                 }
                 __syncthreads();  // sx is rewritten by the next column block or tile
             }
@@ -634,7 +705,20 @@ __global__ void __launch_bounds__(128) conv_pool_solo_tc_kernel(const bf16 *__re
                 for (int c = 0; c < 16; c++) o[c] = __float2bfloat16_rn(z[c]);
                 *reinterpret_cast<uint4 *>(dst + c0) = *reinterpret_cast<const uint4 *>(o);
                 *reinterpret_cast<uint4 *>(dst + c0 + 8) = *reinterpret_cast<const uint4 *>(o + 8);
+                if constexpr (kMode == kTrain) {
+                    uint32_t kk[4];
+#pragma unroll
+                    for (int j = 0; j < 4; j++) {
+                        kk[j] = 0;
+#pragma unroll
+                        for (int e = 0; e < 4; e++)
+                            kk[j] |= (((k1 >> (4 * j + e)) & 1u) | (((k2 >> (4 * j + e)) & 1u) << 1)) << (8 * e);
+                    }
+                    *reinterpret_cast<uint4 *>(idx + ((b * PW + py) * PW + px) * COUT + c0) =
+                        make_uint4(kk[0], kk[1], kk[2], kk[3]);
+                }
             }
+        }
         }
     };
 
@@ -656,7 +740,8 @@ __global__ void __launch_bounds__(128) conv_pool_solo_tc_kernel(const bf16 *__re
             for (int kk = 0; kk < NK16; kk++) {
                 const uint64_t ad = tc::smem_desc(a_addr + kk * 256, 128, SBO);
                 const uint64_t bd = tc::smem_desc(b_addr + kk * 256, 128, SBO);
-                tc::mma_bf16(tmem, ad, bd, kIdesc, kk > 0 ? 1u : 0u);
+                tc::mma_bf16(tmem + (uint32_t)(kk / kTapSteps * COUT), ad, bd, kIdesc,
+                             kk % kTapSteps > 0 ? 1u : 0u);
             }
             tc::mma_commit(bar0);
         }
@@ -685,6 +770,129 @@ __global__ void __launch_bounds__(128) conv_pool_solo_tc_kernel(const bf16 *__re
     if (warp == 0) tc::tmem_dealloc(tmem, kCols);
 }
 
+// Layer 0 of a training pass: conv 3x3 (1 -> 8, pad 1) + bias + ReLU + 2x2 max-pool
+// from the FP32 snippets, keeping the ReLU outputs z (FP32 [B][64][64][8]) and the
+// pool's argmax.  One K = 16 MMA per 128-pixel tile (two image rows; the nine taps
+// and seven zeros, eight channels and eight zeros), so that z has the tensor
+// cores' summation order; the tile's rows are built by the threads, one pixel each.
+// Bound by the 33 MB of z per 256 snippets; small CTAs, 16 per SM, hide the chain of
+// gather, MMA and epilogue.
+__global__ void __launch_bounds__(128) conv0_train_tc_kernel(const float *__restrict__ x, int B,
+                                                             const bf16 *__restrict__ W0,
+                                                             const float *__restrict__ b0,
+                                                             bf16 *__restrict__ a0,
+                                                             float *__restrict__ z_out,
+                                                             uint8_t *__restrict__ idx, int *err) {
+    constexpr int C = 8;
+    constexpr uint32_t SBO = 256, kIdesc = tc::idesc_bf16(128, 16);
+    __shared__ __align__(1024) uint8_t sA[128 * 32];
+    __shared__ __align__(128) uint8_t sB[16 * 32];
+    __shared__ __align__(8) uint64_t bar;
+    __shared__ uint32_t tmem_slot;
+    __shared__ float sbias[C];
+    __shared__ __align__(16) float sx[2][16][C];  // odd rows' column-pair maxima
+    __shared__ uint32_t sk[2][16];
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    if (warp == 0) tc::tmem_alloc(tc::smem_u32(&tmem_slot), 32);
+    if (tid == 0) tc::mbar_init1(tc::smem_u32(&bar));
+    if (tid < C) sbias[tid] = b0[tid];
+    if (tid < 32) {  // weights: row n < 8, half q of K
+        const int n = tid & 15, q = tid >> 4;
+        uint4 v = make_uint4(0u, 0u, 0u, 0u);
+        if (n < C) v = __ldg(reinterpret_cast<const uint4 *>(W0 + n * kpad(0)) + q);
+        *reinterpret_cast<uint4 *>(sB + (n >> 3) * SBO + q * 128 + (n & 7) * 16) = v;
+    }
+    tc::fence_before();
+    __syncthreads();
+    tc::fence_after();
+    const uint32_t tmem = tmem_slot, bar0 = tc::smem_u32(&bar);
+    const uint64_t ad = tc::smem_desc(tc::smem_u32(sA), 128, SBO), bd = tc::smem_desc(tc::smem_u32(sB), 128, SBO);
+    const int64_t ntiles = (int64_t)B * kS * kS / 128;
+    uint32_t ph = 0;
+    bool ok = true, pend = false;
+    for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+        const int64_t b = tile / (kS * kS / 128);
+        const int y0 = 2 * (int)(tile - b * (kS * kS / 128));
+        const int y = y0 + (warp >> 1), xc = (warp & 1) * 32 + lane;
+        const float *img = x + b * kS * kS;
+        __align__(16) bf16 row[16];
+#pragma unroll
+        for (int t = 0; t < 16; t++) row[t] = __float2bfloat16_rn(0.0f);
+#pragma unroll
+        for (int t = 0; t < 9; t++) {
+            const int yy = y + t / 3 - 1, xx = xc + t % 3 - 1;
+            if ((unsigned)yy < (unsigned)kS && (unsigned)xx < (unsigned)kS)
+                row[t] = __float2bfloat16_rn(__ldg(img + yy * kS + xx));
+        }
+        uint8_t *dst = sA + (tid >> 3) * SBO + (tid & 7) * 16;
+        *reinterpret_cast<uint4 *>(dst) = *reinterpret_cast<const uint4 *>(row);
+        *reinterpret_cast<uint4 *>(dst + 128) = *reinterpret_cast<const uint4 *>(row + 8);
+        tc::fence_proxy_async();
+        tc::fence_before();
+        __syncthreads();
+        tc::fence_after();
+        if (tid == 0) {
+            tc::mma_bf16(tmem, ad, bd, kIdesc, 0u);
+            tc::mma_commit(bar0);
+        }
+        pend = true;
+        const bool done = tc::mbar_wait_bounded(bar0, ph, kConvBudget);
+        if (!__syncthreads_and(done)) {
+            ok = false;
+            break;
+        }
+        ph ^= 1u;
+        pend = false;
+        tc::fence_after();
+        float v[16], z[C];
+        tc::tmem_ld16(tmem + ((uint32_t)(warp * 32) << 16), v);
+        uint32_t k1 = 0, k2 = 0;
+#pragma unroll
+        for (int c = 0; c < C; c++) z[c] = fmaxf(v[c] + sbias[c], 0.0f);
+        float4 *o = reinterpret_cast<float4 *>(z_out + ((b * kS + y) * kS + xc) * C);
+        o[0] = make_float4(z[0], z[1], z[2], z[3]);
+        o[1] = make_float4(z[4], z[5], z[6], z[7]);
+#pragma unroll
+        for (int c = 0; c < C; c++) {
+            const float r = __shfl_xor_sync(0xffffffffu, z[c], 1);
+            k1 |= (r > z[c] ? 1u : 0u) << c;
+            z[c] = fmaxf(z[c], r);
+        }
+        if (warp >= 2 && (lane & 1) == 0) {
+            float4 *q = reinterpret_cast<float4 *>(sx[warp & 1][lane >> 1]);
+            q[0] = make_float4(z[0], z[1], z[2], z[3]);
+            q[1] = make_float4(z[4], z[5], z[6], z[7]);
+            sk[warp & 1][lane >> 1] = k1;
+        }
+        __syncthreads();
+        if (warp < 2 && (lane & 1) == 0) {
+            const float *q = sx[warp][lane >> 1];
+            const uint32_t kb = sk[warp][lane >> 1];
+            __align__(16) bf16 h[C];
+            uint32_t kk[2] = {0u, 0u};
+#pragma unroll
+            for (int c = 0; c < C; c++) {
+                const bool low = q[c] > z[c];
+                h[c] = __float2bfloat16_rn(fmaxf(z[c], q[c]));
+                k2 = low ? 2u + ((kb >> c) & 1u) : ((k1 >> c) & 1u);
+                kk[c >> 2] |= k2 << (8 * (c & 3));
+            }
+            const int64_t pix = (b * (kS / 2) + y0 / 2) * (kS / 2) + (xc >> 1);
+            *reinterpret_cast<uint4 *>(a0 + pix * C) = *reinterpret_cast<const uint4 *>(h);
+            *reinterpret_cast<uint2 *>(idx + pix * C) = make_uint2(kk[0], kk[1]);
+        }
+        // sA and the accumulator are rewritten after the next tile's barriers, sx after its
+        // first one
+    }
+    if (!ok) {
+        if (tid == 0) atomicExch(err, 1);
+        if (pend) (void)tc::mbar_wait_bounded(bar0, ph, kConvBudget);
+    }
+    tc::fence_before();
+    __syncthreads();
+    if (warp == 0) tc::tmem_dealloc(tmem, 32);
+}
+
 template <int CIN, int COUT>
 constexpr int conv_pool_solo_smem() {
     return 128 * ((9 * CIN + 15) / 16) * 2 * 16 + COUT * ((9 * CIN + 15) / 16) * 2 * 16 + 8 + 16;
@@ -698,17 +906,16 @@ struct gsp_ranker_s {
     float *params = nullptr, *grads = nullptr, *m = nullptr, *v = nullptr;
     int64_t step = 0;
     // packed bf16 weights
-    bf16 *W[kLayers] = {}, *WT[kLayers] = {}, *W4 = nullptr, *W4T = nullptr;
+    bf16 *W[kLayers] = {}, *WG[kLayers] = {}, *W4 = nullptr, *W4T = nullptr;
     // activations
-    bf16 *col[kLayers] = {}, *colT[kLayers] = {}, *a[kLayers] = {};
+    bf16 *a[kLayers] = {};
     float *z[kLayers] = {};
     uint8_t *idx[kLayers] = {};
     float *z4 = nullptr, *z5 = nullptr, *g5 = nullptr, *ga3 = nullptr, *loss = nullptr;
     bf16 *a4 = nullptr, *g4 = nullptr, *g4T = nullptr, *a3T = nullptr;
     // backward scratch
-    bf16 *gz[kLayers] = {}, *gzT[kLayers] = {};
+    bf16 *gz[kLayers] = {};
     float *ga[kLayers] = {};    // gradient w.r.t. the pooled output of layer l
-    float *dcol = nullptr, *dW = nullptr;
     float *fc1_part = nullptr;  // [kFc1Split][max_batch][kHid] partial products of fc1
     int *err = nullptr;
     std::vector<void *> allocs;
@@ -749,8 +956,8 @@ int blocks_for(int64_t n, int threads = 256) {
 
 cudaError_t pack(gsp_ranker_s *r, cudaStream_t s) {
     RK_LAUNCH((pack_kernel<<<blocks_for((int64_t)kHid * kFc), 256, 0, s>>>(
-        r->params, r->off.w[0], r->off.w[1], r->off.w[2], r->off.w[3], r->W[0], r->WT[0], r->W[1],
-        r->WT[1], r->W[2], r->WT[2], r->W4, r->W4T)));
+        r->params, r->off.w[0], r->off.w[1], r->off.w[2], r->off.w[3], r->W[0], r->W[1], r->W[2],
+        r->WG[1], r->WG[2], r->W4, r->W4T)));
     return cudaSuccess;
 }
 
@@ -788,18 +995,17 @@ cudaError_t conv_ctas_per_sm(Kern kern, int smem, int cols, int *out) {
     return cudaSuccess;
 }
 
-template <int CIN, int COUT, int SIDE>
-cudaError_t launch_conv_pool_solo(gsp_ranker_s *r, const bf16 *act, int n, const bf16 *W,
-                                  const float *bias, bf16 *out, cudaStream_t s, bool dependent) {
+template <int CIN, int COUT, int SIDE, ConvMode kMode>
+cudaError_t launch_conv(gsp_ranker_s *r, const bf16 *act, int n, const bf16 *W, const float *bias,
+                        bf16 *out, float *z, uint8_t *idx, int nz, cudaStream_t s) {
     constexpr int smem = conv_pool_solo_smem<CIN, COUT>();
+    auto kern = conv_pool_solo_tc_kernel<CIN, COUT, SIDE, kMode>;
     static int blocks_per_sm = 0;
     if (blocks_per_sm == 0) {
-        cudaError_t e = conv_ctas_per_sm(conv_pool_solo_tc_kernel<CIN, COUT, SIDE>, smem, COUT,
-                                         &blocks_per_sm);
+        cudaError_t e = conv_ctas_per_sm(kern, smem, (int)conv_tmem_cols(COUT, kMode), &blocks_per_sm);
         if (e != cudaSuccess) return e;
     } else {
-        cudaError_t e = gsp::ensure_kernel_smem(
-            reinterpret_cast<const void *>(conv_pool_solo_tc_kernel<CIN, COUT, SIDE>), smem, true);
+        cudaError_t e = gsp::ensure_kernel_smem(reinterpret_cast<const void *>(kern), smem, true);
         if (e != cudaSuccess) return e;
     }
     int dev = 0, sms = 0;
@@ -808,57 +1014,35 @@ cudaError_t launch_conv_pool_solo(gsp_ranker_s *r, const bf16 *act, int n, const
     if (e != cudaSuccess) return e;
     const int64_t ntiles = (int64_t)n * SIDE * SIDE / 128;
     const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(ntiles, (int64_t)sms * blocks_per_sm));
-    if (dependent) {
-        e = gsp::launch_dependent(conv_pool_solo_tc_kernel<CIN, COUT, SIDE>, dim3(grid), dim3(128),
-                                  (size_t)smem, s, act, n, W, bias, out, r->err);
-        if (e != cudaSuccess) return e;
-        r->launches++;
-        return cudaSuccess;
-    }
-    RK_LAUNCH((conv_pool_solo_tc_kernel<CIN, COUT, SIDE><<<grid, 128, smem, s>>>(act, n, W, bias, out,
-                                                                               r->err)));
+    // a programmatic dependent of the kernel before it (it waits in wait_prior_grid)
+    e = gsp::launch_dependent(kern, dim3(grid), dim3(128), (size_t)smem, s, act, n, W, bias, out, z, idx,
+                              nz, r->err);
+    if (e != cudaSuccess) return e;
+    r->launches++;
     return cudaSuccess;
 }
 
-// Forward pass of n snippets (FP32 [n][64][64]); logits into r->z5.  A
-// training pass keeps what the backward pass needs (im2col matrices,
-// pre-activations, pool argmaxes); an inference pass runs each conv layer as
-// one fused conv + bias + ReLU + pool kernel.
+// Forward pass of n snippets (FP32 [n][64][64]); logits into r->z5.  Each conv
+// layer is one fused conv + bias + ReLU + pool kernel; in a training pass they
+// also keep the ReLU outputs and the pool argmaxes.
 cudaError_t forward(gsp_ranker_s *r, const float *x, int n, bool train, cudaStream_t s) {
-    for (int l = 0; l < kLayers; l++) {
-        const int H = side_of(l), Cin = cin_of(l), Cout = cout_of(l), Kp = kpad(l);
-        const int64_t P = (int64_t)n * H * H;
-        (void)Cin;
-        if (!train) {
-            cudaError_t e = cudaSuccess;
-            if (l == 0)
-                RK_LAUNCH((conv0_pool_kernel<<<blocks_for(P / 8), 256, 0, s>>>(
-                    x, n, r->W[0], r->params + r->off.b[0], r->a[0])));
-            else if (l == 1)
-                e = launch_conv_pool_solo<8, 16, 32>(r, r->a[0], n, r->W[1], r->params + r->off.b[1],
-                                                     r->a[1], s, true);
-            else
-                e = launch_conv_pool_solo<16, 32, 16>(r, r->a[1], n, r->W[2], r->params + r->off.b[2],
-                                                      r->a[2], s, true);
-            if (e != cudaSuccess) return e;
-            continue;
-        }
-        if (l == 0)
-            RK_LAUNCH((im2col_kernel<float, 1><<<blocks_for(P), 256, 0, s>>>(x, n, H, r->col[0])));
-        else if (l == 1)
-            RK_LAUNCH((im2col_kernel<bf16, 8><<<blocks_for(P), 256, 0, s>>>(r->a[0], n, H, r->col[1])));
-        else
-            RK_LAUNCH((im2col_kernel<bf16, 16><<<blocks_for(P), 256, 0, s>>>(r->a[1], n, H, r->col[2])));
-        cudaError_t e = gemm(r, r->col[l], Kp, r->W[l], Kp, r->z[l], Cout, nullptr, 0, (int)P, Cout,
-                             Kp, r->params + r->off.b[l], true, 1, s);
-        if (e != cudaSuccess) return e;
-        if (l == 0)
-            RK_LAUNCH((pool_kernel<8><<<blocks_for(P / 4), 256, 0, s>>>(r->z[0], n, H, r->a[0], r->idx[0])));
-        else if (l == 1)
-            RK_LAUNCH((pool_kernel<16><<<blocks_for(P / 4), 256, 0, s>>>(r->z[1], n, H, r->a[1], r->idx[1])));
-        else
-            RK_LAUNCH((pool_kernel<32><<<blocks_for(P / 4), 256, 0, s>>>(r->z[2], n, H, r->a[2], r->idx[2])));
+    const int grid0 = blocks_for((int64_t)n * kS * kS / 8);
+    const float *const b1 = r->params + r->off.b[1], *const b2 = r->params + r->off.b[2];
+    cudaError_t e;
+    if (train) {
+        RK_LAUNCH((conv0_train_tc_kernel<<<(int)std::min<int64_t>((int64_t)n * kS * kS / 128, 152 * 16), 128, 0,
+                                           s>>>(x, n, r->W[0], r->params + r->off.b[0], r->a[0], r->z[0],
+                                                r->idx[0], r->err)));
+        e = launch_conv<8, 16, 32, kTrain>(r, r->a[0], n, r->W[1], b1, r->a[1], r->z[1], r->idx[1], 0, s);
+        if (e == cudaSuccess)
+            e = launch_conv<16, 32, 16, kTrain>(r, r->a[1], n, r->W[2], b2, r->a[2], r->z[2], r->idx[2], 0, s);
+    } else {
+        RK_LAUNCH((conv0_pool_kernel<<<grid0, 256, 0, s>>>(x, n, r->W[0], r->params + r->off.b[0], r->a[0])));
+        e = launch_conv<8, 16, 32, kInfer>(r, r->a[0], n, r->W[1], b1, r->a[1], nullptr, nullptr, 0, s);
+        if (e == cudaSuccess)
+            e = launch_conv<16, 32, 16, kInfer>(r, r->a[1], n, r->W[2], b2, r->a[2], nullptr, nullptr, 0, s);
     }
+    if (e != cudaSuccess) return e;
     // fc1 (K = 2048) as a deterministic split-K product: enough K chunks for a
     // CTA per SM even at one column block, at least four 64-wide steps each;
     // the chunks' partial products are summed in order by fc1_finish_kernel
@@ -869,82 +1053,67 @@ cudaError_t forward(gsp_ranker_s *r, const float *x, int n, bool train, cudaStre
     const int want = std::max(1, std::min(kFc1Split, std::min(kFc / (4 * 64), nsm / mt)));
     const int64_t zs = (int64_t)r->max_batch * kHid;
     int used = 1;
-    // in an inference pass each kernel after the first is launched as a
+    // each kernel after the first is launched as a
     // programmatic dependent of the one before (its blocks are scheduled while
     // that kernel drains and wait for its output in wait_prior_grid)
-    cudaError_t e = gsp::launch_gemm_bf16(r->a[2], kFc, r->W4, kFc, r->fc1_part, kHid, nullptr, 0, n,
-                                          kHid, kFc, nullptr, false, want, r->err, s, zs, &used,
-                                          !train);
+    e = gsp::launch_gemm_bf16(r->a[2], kFc, r->W4, kFc, r->fc1_part, kHid, nullptr, 0, n, kHid, kFc,
+                              nullptr, false, want, r->err, s, zs, &used, true);
     if (e != cudaSuccess) return e;
     r->launches++;
-    if (!train) {
-        e = gsp::launch_dependent(fc1_finish_kernel, dim3(blocks_for((int64_t)n * kHid)), dim3(256),
-                                  0, s, (const float *)r->fc1_part, used, zs, n,
-                                  (const float *)(r->params + r->off.b[3]), r->z4, r->a4);
-        if (e == cudaSuccess)
-            e = gsp::launch_dependent(fc2_kernel, dim3((2 * n + 127) / 128), dim3(128), 0, s,
-                                      (const bf16 *)r->a4, (const float *)(r->params + r->off.w[4]),
-                                      (const float *)(r->params + r->off.b[4]), n, r->z5);
-        if (e != cudaSuccess) return e;
-        r->launches += 2;
-        return cudaSuccess;
-    }
-    RK_LAUNCH((fc1_finish_kernel<<<blocks_for((int64_t)n * kHid), 256, 0, s>>>(
-        r->fc1_part, used, zs, n, r->params + r->off.b[3], r->z4, r->a4)));
-    RK_LAUNCH((fc2_kernel<<<(2 * n + 127) / 128, 128, 0, s>>>(r->a4, r->params + r->off.w[4],
-                                                              r->params + r->off.b[4], n, r->z5)));
+    e = gsp::launch_dependent(fc1_finish_kernel, dim3(blocks_for((int64_t)n * kHid)), dim3(256), 0, s,
+                              (const float *)r->fc1_part, used, zs, n,
+                              (const float *)(r->params + r->off.b[3]), r->z4, r->a4);
+    if (e == cudaSuccess)
+        e = gsp::launch_dependent(fc2_kernel, dim3((2 * n + 127) / 128), dim3(128), 0, s,
+                                  (const bf16 *)r->a4, (const float *)(r->params + r->off.w[4]),
+                                  (const float *)(r->params + r->off.b[4]), n, r->z5);
+    if (e != cudaSuccess) return e;
+    r->launches += 2;
     return cudaSuccess;
 }
 
 // Loss, gradients (into r->grads, the oracle's layout) and one Adam step.
-cudaError_t backward(gsp_ranker_s *r, const int32_t *labels, int n, float lr, cudaStream_t s) {
+cudaError_t backward(gsp_ranker_s *r, const float *x, const int32_t *labels, int n, float lr,
+                     cudaStream_t s) {
     const int n8 = round8(n);
     cudaError_t e = cudaMemsetAsync(r->grads, 0, (size_t)r->off.total * sizeof(float), s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(r->g4T, 0, (size_t)kHid * n8 * sizeof(bf16), s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(r->a3T, 0, (size_t)kFc * n8 * sizeof(bf16), s);
+    if (n8 != n) {  // the padding columns of the transposed operands
+        if (e == cudaSuccess) e = cudaMemsetAsync(r->g4T, 0, (size_t)kHid * n8 * sizeof(bf16), s);
+        if (e == cudaSuccess) e = cudaMemsetAsync(r->a3T, 0, (size_t)kFc * n8 * sizeof(bf16), s);
+    }
     if (e != cudaSuccess) return e;
+    float *const gr = r->grads;
+    const Offsets &o = r->off;
     RK_LAUNCH((loss_kernel<<<1, 256, 0, s>>>(r->z5, labels, n, r->g5, r->loss)));
-    RK_LAUNCH((fc2_back_kernel<<<std::min(n, 152), kHid, 0, s>>>(
-        r->g5, r->a4, r->params + r->off.w[4], r->z4, n, r->grads + r->off.w[4],
-        r->grads + r->off.b[4], r->g4, r->g4T, n8, r->grads + r->off.b[3])));
+    RK_LAUNCH((fc2_back_kernel<<<std::min((n + 3) / 4, 152), kHid, 0, s>>>(
+        r->g5, r->a4, r->params + o.w[4], r->z4, n, gr + o.w[4], gr + o.b[4], r->g4, r->g4T, n8,
+        gr + o.b[3])));
     {
         dim3 grid((unsigned)((n + 31) / 32), (unsigned)(kFc / 32));
         RK_LAUNCH((transpose_kernel<<<grid, dim3(32, 8), 0, s>>>(r->a[2], kFc, n, kFc, r->a3T, n8)));
     }
-    e = gemm(r, r->g4T, n8, r->a3T, n8, r->grads + r->off.w[3], kFc, nullptr, 0, kHid, kFc, n8,
-             nullptr, false, 1, s);
+    e = gemm(r, r->g4T, n8, r->a3T, n8, gr + o.w[3], kFc, nullptr, 0, kHid, kFc, n8, nullptr, false, 1, s);
     if (e == cudaSuccess)
         e = gemm(r, r->g4, kHid, r->W4T, kHid, r->ga[2], kFc, nullptr, 0, n, kFc, kHid, nullptr,
                  false, 1, s);
     if (e != cudaSuccess) return e;
-    for (int l = kLayers - 1; l >= 0; l--) {
-        const int H = side_of(l), Cin = cin_of(l), Cout = cout_of(l), Kp = kpad(l);
-        const int64_t P = (int64_t)n * H * H;  // a multiple of 256
-        RK_LAUNCH((pool_back_kernel<<<blocks_for(P * Cout), 256, Cout * sizeof(float), s>>>(
-            r->ga[l], r->idx[l], r->z[l], n, H, Cout, r->gz[l], r->gzT[l], P,
-            r->grads + r->off.b[l])));
-        {
-            dim3 grid((unsigned)((P + 31) / 32), (unsigned)((Kp + 31) / 32));
-            RK_LAUNCH((transpose_kernel<<<grid, dim3(32, 8), 0, s>>>(r->col[l], Kp, P, Kp,
-                                                                      r->colT[l], P)));
-        }
-        e = cudaMemsetAsync(r->dW, 0, (size_t)Cout * Kp * sizeof(float), s);
-        if (e != cudaSuccess) return e;
-        const int ksteps = (int)(P / 64);
-        const int splitk = std::max(1, std::min(ksteps, 4 * 152 / std::max(1, (Kp + 127) / 128)));
-        e = gemm(r, r->gzT[l], P, r->colT[l], P, r->dW, Kp, nullptr, 0, Cout, Kp, (int)P, nullptr,
-                 false, splitk, s);
-        if (e != cudaSuccess) return e;
-        RK_LAUNCH((unpack_conv_grad_kernel<<<(Cout * Cin * 9 + 255) / 256, 256, 0, s>>>(
-            r->dW, Cin, Cout, Kp, r->grads + r->off.w[l])));
-        if (l > 0) {
-            e = gemm(r, r->gz[l], Cout, r->WT[l], round8(Cout), r->dcol, Kp, nullptr, 0, (int)P, Kp,
-                     Cout, nullptr, false, 1, s);
-            if (e != cudaSuccess) return e;
-            RK_LAUNCH((col2im_kernel<<<blocks_for(P * Cin), 256, 0, s>>>(r->dcol, n, H, Cin, Kp,
-                                                                          r->ga[l - 1])));
-        }
-    }
+    // per layer: back through pool and ReLU, weight gradient, input gradient
+    RK_LAUNCH((pool_back_kernel<32><<<blocks_for((int64_t)n * 8 * 8 * 4), 256, 0, s>>>(
+        r->ga[2], r->idx[2], r->a[2], n, 16, r->gz[2], gr + o.b[2])));
+    e = launch_conv<32, kGradRows, 16, kGrad>(r, r->gz[2], n, r->WG[2], nullptr, nullptr, r->ga[1], nullptr, 16, s);
+    if (e != cudaSuccess) return e;
+    RK_LAUNCH((conv_dw_kernel<bf16, 16, 32, 16><<<std::min(n, 912), 256, 0, s>>>(
+        r->a[1], n, r->ga[2], r->idx[2], r->a[2], gr + o.w[2])));
+    RK_LAUNCH((pool_back_kernel<16><<<blocks_for((int64_t)n * 16 * 16 * 2), 256, 0, s>>>(
+        r->ga[1], r->idx[1], r->a[1], n, 32, r->gz[1], gr + o.b[1])));
+    e = launch_conv<16, kGradRows, 32, kGrad>(r, r->gz[1], n, r->WG[1], nullptr, nullptr, r->ga[0], nullptr, 8, s);
+    if (e != cudaSuccess) return e;
+    RK_LAUNCH((conv_dw_kernel<bf16, 8, 16, 32><<<std::min(2 * n, 912), 256, 0, s>>>(
+        r->a[0], n, r->ga[1], r->idx[1], r->a[1], gr + o.w[1])));
+    RK_LAUNCH((pool_back_kernel<8><<<blocks_for((int64_t)n * 32 * 32), 256, 0, s>>>(
+        r->ga[0], r->idx[0], r->a[0], n, 64, r->gz[0], gr + o.b[0])));
+    RK_LAUNCH((conv_dw_kernel<float, 1, 8, 64><<<std::min(4 * n, 912), 256, 0, s>>>(
+        x, n, r->ga[0], r->idx[0], r->a[0], gr + o.w[0])));
     r->step++;
     const double c1 = 1.0 - std::pow(0.9, (double)r->step);
     const double c2 = 1.0 - std::pow(0.999, (double)r->step);
@@ -1446,20 +1615,15 @@ gsp_status gsp_ranker_create(gsp_ranker_t *out, int32_t max_batch, uint64_t seed
               ralloc(r, &r->g5, (size_t)Bm * 2) && ralloc(r, &r->g4, (size_t)Bm * kHid) &&
               ralloc(r, &r->g4T, (size_t)kHid * B8) && ralloc(r, &r->a3T, (size_t)kFc * B8) &&
               ralloc(r, &r->loss, 1) && ralloc(r, &r->err, 1);
-    size_t dcol = 0, dw = 0;
     for (int l = 0; ok && l < kLayers; l++) {
         const int H = side_of(l), Cout = cout_of(l), Kp = kpad(l);
         const int64_t P = (int64_t)Bm * H * H;
-        ok = ralloc(r, &r->W[l], (size_t)Cout * Kp) && ralloc(r, &r->WT[l], (size_t)Kp * round8(Cout)) &&
-             ralloc(r, &r->col[l], (size_t)P * Kp) && ralloc(r, &r->colT[l], (size_t)P * Kp) &&
+        ok = ralloc(r, &r->W[l], (size_t)Cout * Kp) && ralloc(r, &r->WG[l], (size_t)kGradRows * 9 * Cout) &&
              ralloc(r, &r->z[l], (size_t)P * Cout) && ralloc(r, &r->a[l], (size_t)P / 4 * Cout) &&
              ralloc(r, &r->idx[l], (size_t)P / 4 * Cout) && ralloc(r, &r->gz[l], (size_t)P * Cout) &&
-             ralloc(r, &r->gzT[l], (size_t)P * Cout) && ralloc(r, &r->ga[l], (size_t)P / 4 * Cout);
-        if (l > 0) dcol = std::max(dcol, (size_t)P * Kp);
-        dw = std::max(dw, (size_t)Cout * Kp);
+             ralloc(r, &r->ga[l], (size_t)P / 4 * Cout);
     }
-    ok = ok && ralloc(r, &r->dcol, dcol) && ralloc(r, &r->dW, dw) &&
-         ralloc(r, &r->fc1_part, (size_t)kFc1Split * Bm * kHid);
+    ok = ok && ralloc(r, &r->fc1_part, (size_t)kFc1Split * Bm * kHid);
     if (!ok) {
         free_ranker(r);
         return GSP_ERR_OOM;
@@ -1540,7 +1704,7 @@ gsp_status gsp_ranker_train_step(gsp_ranker_t r, const float *d_x, const int32_t
     cudaStream_t s = (cudaStream_t)stream;
     r->launches = 0;
     cudaError_t e = forward(r, d_x, n, true, s);
-    if (e == cudaSuccess) e = backward(r, d_labels, n, lr, s);
+    if (e == cudaSuccess) e = backward(r, d_x, d_labels, n, lr, s);
     r->last_n = n;
     r->last_pass = 2;
     if (e == cudaSuccess && d_loss)
