@@ -57,67 +57,75 @@ __global__ void __launch_bounds__(256) ingest_transpose_kernel(const uint8_t *__
 }
 
 // The same with 16-byte global accesses (pointers and strides 16-byte
-// aligned) on 256 (time) x 64 (channel) tiles: thread (r, q) loads bytes
-// [16q, 16q + 16) of time rows r, r + 64, r + 128, r + 192 into 4-byte words of a
-// padded tile (17 words per row); thread (c, q) then gathers byte c of the
-// 16-sample groups q, q + 4, q + 8, q + 12 into 16-byte stores of channel row c.
-// Four loads and four stores per thread keep more bytes in flight.  Edge
-// tiles fall back to byte accesses.
+// aligned) on 256 (time) x 64 (channel) tiles.  Thread (r, q) loads bytes
+// [16q, 16q + 16) of time rows 4r .. 4r + 3 and transposes their 4 x 4 byte blocks in
+// registers (8 byte permutes per 16 bytes): 16 words of four samples, one per
+// channel, into the shared tile [channel][time].  Each half warp then reads 256
+// samples of a channel as 16-byte words and stores them, 256 contiguous bytes.
+// The tile's word column is XORed with 8 times the channel group, which keeps both
+// sides free of bank conflicts.  About 1.1 instructions per byte (four when each
+// byte was gathered from shared memory on its own).  4096 x 262144 samples: 458 ->
+// 346 us (6.2 TB/s of the 6.8 measured).  Edge tiles fall back to byte accesses.
 constexpr int kTileT16 = 256;
 
 __global__ void __launch_bounds__(256) ingest_transpose16_kernel(const uint8_t *__restrict__ in,
                                                                  int64_t in_stride, int64_t N,
                                                                  int C, uint8_t *__restrict__ out,
                                                                  int64_t out_stride) {
-    __shared__ uint32_t tile[kTileT16][17];
+    __shared__ __align__(16) uint32_t tile[kTile][kTileT16 / 4];
     const int64_t t0 = (int64_t)blockIdx.x * kTileT16;
     const int c0 = blockIdx.y * kTile;
-    const int q = threadIdx.x & 3;
-#pragma unroll
-    for (int i = 0; i < kTileT16 / 64; i++) {
-        const int r = (threadIdx.x >> 2) + 64 * i;
-        const int64_t t = t0 + r;
+    {
+        const int q = threadIdx.x & 3, r = threadIdx.x >> 2;
         const int c = c0 + 16 * q;
-        uint4 v = make_uint4(0u, 0u, 0u, 0u);
-        if (t < N) {
+        uint32_t v[4][4];
+#pragma unroll
+        for (int i = 0; i < 4; i++) {
+            const int64_t t = t0 + 4 * r + i;
             const uint8_t *src = in + t * in_stride + c;
-            if (c + 15 < C) {
-                v = __ldg(reinterpret_cast<const uint4 *>(src));
-            } else {
-                uint32_t w[4] = {0u, 0u, 0u, 0u};
-                for (int k = 0; k < 16; k++)
-                    if (c + k < C) w[k >> 2] |= (uint32_t)__ldg(src + k) << (8 * (k & 3));
-                v = make_uint4(w[0], w[1], w[2], w[3]);
+            uint4 x = make_uint4(0u, 0u, 0u, 0u);
+            if (t < N) {
+                if (c + 15 < C) {
+                    x = __ldcs(reinterpret_cast<const uint4 *>(src));
+                } else {
+                    uint32_t w[4] = {0u, 0u, 0u, 0u};
+                    for (int k = 0; k < 16; k++)
+                        if (c + k < C) w[k >> 2] |= (uint32_t)__ldg(src + k) << (8 * (k & 3));
+                    x = make_uint4(w[0], w[1], w[2], w[3]);
+                }
             }
+            v[i][0] = x.x;
+            v[i][1] = x.y;
+            v[i][2] = x.z;
+            v[i][3] = x.w;
         }
-        tile[r][4 * q + 0] = v.x;
-        tile[r][4 * q + 1] = v.y;
-        tile[r][4 * q + 2] = v.z;
-        tile[r][4 * q + 3] = v.w;
+#pragma unroll
+        for (int k = 0; k < 4; k++) {
+            const uint32_t lo01 = __byte_perm(v[0][k], v[1][k], 0x5140), lo23 = __byte_perm(v[2][k], v[3][k], 0x5140);
+            const uint32_t hi01 = __byte_perm(v[0][k], v[1][k], 0x7362), hi23 = __byte_perm(v[2][k], v[3][k], 0x7362);
+            const int col = r ^ (8 * q);
+            tile[16 * q + 4 * k + 0][col] = __byte_perm(lo01, lo23, 0x5410);
+            tile[16 * q + 4 * k + 1][col] = __byte_perm(lo01, lo23, 0x7632);
+            tile[16 * q + 4 * k + 2][col] = __byte_perm(hi01, hi23, 0x5410);
+            tile[16 * q + 4 * k + 3][col] = __byte_perm(hi01, hi23, 0x7632);
+        }
     }
     __syncthreads();
-    const int cl = threadIdx.x >> 2;   // channel inside the tile
-    const int c = c0 + cl;
-    if (c >= C) return;
-    const uint32_t sh = 8u * (uint32_t)(cl & 3);
+    const int m = threadIdx.x & 15;        // 16-sample group inside the tile
+    const int64_t t = t0 + 16 * m;
 #pragma unroll
-    for (int j = 0; j < kTileT16 / 64; j++) {
-        const int grp = q + 4 * j;       // 16-sample group inside the tile
-        const int64_t t = t0 + 16 * grp;
-        uint32_t w[4];
-#pragma unroll
-        for (int g = 0; g < 4; g++) {
-            uint32_t b[4];
-#pragma unroll
-            for (int k = 0; k < 4; k++) b[k] = (tile[16 * grp + 4 * g + k][cl >> 2] >> sh) & 0xffu;
-            w[g] = b[0] | (b[1] << 8) | (b[2] << 16) | (b[3] << 24);
-        }
+    for (int j = 0; j < 4; j++) {
+        const int cl = (threadIdx.x >> 4) + 16 * j;  // channel inside the tile
+        const int c = c0 + cl;
+        if (c >= C) continue;
+        const uint4 w = *reinterpret_cast<const uint4 *>(&tile[cl][(4 * m) ^ (8 * (cl >> 4))]);
         uint8_t *dst = out + (int64_t)c * out_stride + t;
         if (t + 15 < N) {
-            *reinterpret_cast<uint4 *>(dst) = make_uint4(w[0], w[1], w[2], w[3]);
+            __stcs(reinterpret_cast<uint4 *>(dst), w);
         } else {
+            const uint32_t b[4] = {w.x, w.y, w.z, w.w};
             for (int k = 0; k < 16; k++)
-                if (t + k < N) dst[k] = (uint8_t)(w[k >> 2] >> (8 * (k & 3)));
+                if (t + k < N) dst[k] = (uint8_t)(b[k >> 2] >> (8 * (k & 3)));
         }
     }
 }
