@@ -57,8 +57,9 @@ constexpr int kRawSlot = kChunk * kRawPitch;
 constexpr int kWideSlot = kChunk * kWidePitch;
 // Warps by role (the first two roles: one quarter of the tensor-memory lanes each).
 constexpr int kAWarp = 4;              // 4: write A (warps 0-3 move the rows of D and store it)
-constexpr int kWideWarp = 8;           // 8: widen the channels in turn (8 to 16 warps: within 4%)
-constexpr int kWideWarps = 8;
+constexpr int kWideWarp = 8;           // 11: widen the channels in turn (16.1 ms on a
+                                       // 131072-sample chunk; 8: 16.6, 10: 16.5, 12: 17.0)
+constexpr int kWideWarps = 11;
 constexpr int kMmaWarp = kWideWarp + kWideWarps;  // issue the products (one lane)
 constexpr int kCopyWarp = kMmaWarp + 1;           // 2: copy the channels' windows of the chunks in turn
 constexpr int kCopyWarps = 2;
@@ -82,6 +83,7 @@ struct MmaBeam {
     unsigned long long *bsum;
     int64_t nb_max, Ls, ntiles, item0;
     int ndm, nblk, grp, B, T, rev;
+    int add;  // add to the series that is there (the other channels' sums)
 };
 
 struct MmaArgs {
@@ -199,9 +201,9 @@ __device__ __forceinline__ void widen_channel(uint32_t src, uint32_t dst, uint32
 // their pipelines running on across items.  Warps:
 //   0-3   move the rows of D between frames, store D;
 //   4-7   write A of each chunk;
-//   8-15  widen one channel of each chunk;
-//   16    issues the MMAs (one lane);
-//   17-18 copy the channels' windows of every other chunk each (1-D bulk copies).
+//   8-18  widen the channels in turn;
+//   19    issues the MMAs (one lane);
+//   20-21 copy the channels' windows of every other chunk each (1-D bulk copies).
 // Every wait is bounded: a warp whose wait gives up reports it and leaves its
 // loop; the MMA lane and the copying warp then wait for what they have in flight, and
 // tensor memory is freed after all warps have met.
@@ -337,13 +339,23 @@ __global__ void __launch_bounds__(kThreads, 1) dd_mma_kernel(const __grid_consta
             uint32_t va[16], vb[16];
             // 16 columns at a time: the sums run in 32 bits inside them (x < 2^24,
             // sum i x < 2^31), unless a lane comes to a search block's end there
+            const bool add = bt.add != 0;  // another kernel has left the other channels' sums
             auto store16 = [&](const uint32_t (&v)[16], int c0) {
                 const int tf = 8 * c0 + tau - R;  // the lane's first sample
                 int32_t x[16];
 #pragma unroll
+                for (int i = 0; i < 16; i++) x[i] = (int32_t)(__uint_as_float(v[i]) * 16777216.0f);
+                if (add) {
+                    int32_t o[16];
+#pragma unroll
+                    for (int i = 0; i < 16; i++)
+                        o[i] = (unsigned)(tf + 8 * i) < (unsigned)tlim ? __ldcs(orow + tf + 8 * i) : 0;
+#pragma unroll
+                    for (int i = 0; i < 16; i++) x[i] += o[i];
+                }
+#pragma unroll
                 for (int i = 0; i < 16; i++) {
                     const int t = tf + 8 * i;
-                    x[i] = (int32_t)(__uint_as_float(v[i]) * 16777216.0f);
                     if ((unsigned)t < (unsigned)tlim) __stcs(orow + t, x[i]);
                     x[i] = (unsigned)t < (unsigned)slim ? x[i] : 0;
                 }
@@ -649,9 +661,92 @@ __global__ void __launch_bounds__(kThreads, 1) dd_mma_kernel(const __grid_consta
 
 }  // namespace
 
-bool mma_plan_tables(const int32_t *delays, int ndm, int C, bool rev, MmaTables *t) {
-    const int nblk = (ndm + kKdm - 1) / kKdm, nchunk = (C + kChunk - 1) / kChunk;
-    t->base.assign((size_t)nblk * C, 0);
+namespace {
+
+struct Range {
+    int lo, hi;
+};
+
+// The range of x[i] - y[i] over a block.
+Range range_of(const int32_t *x, const int32_t *y) {
+    int32_t lo = INT32_MAX, hi = INT32_MIN;
+    for (int i = 0; i < kKdm; i++) {
+        const int32_t v = x[i] - y[i];
+        lo = std::min(lo, v);
+        hi = std::max(hi, v);
+    }
+    return Range{lo, hi};
+}
+
+// Delays of block b by position, the 16 trials side by side (loops over them vectorise).
+void block_delays(const int32_t *delays, int ndm, int C, bool rev, int npos, int b, int32_t *dl) {
+    for (int i = 0; i < kKdm; i++) {
+        const int32_t *row = delays + (size_t)std::min(ndm - 1, b * kKdm + i) * C;
+        int32_t *d = dl + i;
+        if (rev)
+            for (int pos = 0; pos < npos; pos++) d[(size_t)pos * kKdm] = row[C - 1 - pos];
+        else
+            for (int pos = 0; pos < npos; pos++) d[(size_t)pos * kKdm] = row[pos];
+    }
+}
+
+// The frames of one block, each followed by visit(position, smallest delay - R) for its
+// positions; R is left at the last frame's.  false if a row moves further than a tile.
+template <typename Visit>
+bool block_frames(const int32_t *dl, int npos, int32_t (&R)[kKdm], std::vector<MmaFrame> *frames,
+                  Visit visit) {
+    for (int i = 0; i < kKdm; i++) R[i] = 0;
+    bool first = true;
+    int rmax = 0;
+    for (int p0 = 0; p0 < npos;) {
+        // centre the frame on the furthest channel whose delays differ from those of
+        // p0 by amounts within 8 samples of each other, with moves of at most 16
+        const int32_t *d0 = dl + (size_t)p0 * kKdm;
+        int best = p0;
+        for (int pos = p0; pos < npos; pos++) {
+            const int32_t *d = dl + (size_t)pos * kKdm;
+            const Range dv = range_of(d, d0), ev = range_of(d, R);
+            if (dv.hi - dv.lo > kMaxShift || (!first && ev.hi - ev.lo > kMaxMove)) break;
+            best = pos;
+        }
+        const int32_t *ref = dl + (size_t)best * kKdm;
+        for (bool more = true; more;) {
+            const int elo = range_of(ref, R).lo;
+            MmaFrame fr;
+            fr.pos = p0;
+            more = false;
+            rmax = 0;
+            for (int i = 0; i < kKdm; i++) {
+                int e = ref[i] - R[i] - elo;
+                if (!first && e > kMaxMove) {  // a steep step: several moves
+                    e = kMaxMove;
+                    more = true;
+                }
+                fr.e[i] = first ? 0 : (uint8_t)e;
+                R[i] += e;
+                rmax = std::max(rmax, (int)R[i]);
+            }
+            fr.rmax = rmax;
+            if (rmax > 8 * kCols) return false;
+            frames->push_back(fr);
+            first = false;
+        }
+        int pos = p0;
+        for (; pos < npos; pos++) {
+            const Range v = range_of(dl + (size_t)pos * kKdm, R);
+            if (v.hi - v.lo > kMaxShift) break;
+            visit(pos, v.lo, rmax);
+        }
+        p0 = pos;
+    }
+    return true;
+}
+
+}  // namespace
+
+bool mma_plan_tables(const int32_t *delays, int ndm, int C, bool rev, int npos, MmaTables *t) {
+    const int nblk = (ndm + kKdm - 1) / kKdm, nchunk = (npos + kChunk - 1) / kChunk;
+    t->base.assign((size_t)nblk * npos, 0);
     t->shift.assign((size_t)nblk * nchunk * kKdm * kChunk, 0);
     t->crmax.assign((size_t)nblk * nchunk, 0);
     t->rlast.assign((size_t)nblk * kKdm, 0);
@@ -659,85 +754,64 @@ bool mma_plan_tables(const int32_t *delays, int ndm, int C, bool rev, MmaTables 
     t->frames.clear();
     t->rmax = 0;
     t->mean_cols_r = 0.0;
-    // a block's delays by position, the 16 trials side by side (loops over them vectorise)
-    std::vector<int32_t> dl((size_t)C * kKdm);
-    struct Range {
-        int lo, hi;
-    };
-    auto range_of = [](const int32_t *x, const int32_t *y) {  // of x[i] - y[i] over the block
-        int32_t lo = INT32_MAX, hi = INT32_MIN;
-        for (int i = 0; i < kKdm; i++) {
-            const int32_t v = x[i] - y[i];
-            lo = std::min(lo, v);
-            hi = std::max(hi, v);
-        }
-        return Range{lo, hi};
-    };
+    std::vector<int32_t> dl((size_t)npos * kKdm);
     for (int b = 0; b < nblk; b++) {
+        block_delays(delays, ndm, C, rev, npos, b, dl.data());
+        int32_t R[kKdm];
+        const bool ok = block_frames(dl.data(), npos, R, &t->frames, [&](int pos, int lo, int rmax) {
+            const int32_t *d = dl.data() + (size_t)pos * kKdm;
+            t->base[(size_t)b * npos + pos] = lo;
+            uint8_t *sh = t->shift.data() + ((size_t)b * nchunk + pos / kChunk) * kKdm * kChunk + pos % kChunk;
+            for (int i = 0; i < kKdm; i++) sh[i * kChunk] = (uint8_t)(d[i] - R[i] - lo);
+            int32_t &cr = t->crmax[(size_t)b * nchunk + pos / kChunk];
+            cr = std::max(cr, rmax);
+            t->mean_cols_r += rmax;
+        });
+        if (!ok) return false;
         for (int i = 0; i < kKdm; i++) {
-            const int32_t *row = delays + (size_t)std::min(ndm - 1, b * kKdm + i) * C;
-            int32_t *d = dl.data() + i;
-            if (rev)
-                for (int pos = 0; pos < C; pos++) d[(size_t)pos * kKdm] = row[C - 1 - pos];
-            else
-                for (int pos = 0; pos < C; pos++) d[(size_t)pos * kKdm] = row[pos];
+            t->rlast[(size_t)b * kKdm + i] = R[i];
+            t->rmax = std::max(t->rmax, (int)R[i]);
         }
-        int32_t R[kKdm] = {};
-        bool first = true;
-        int rmax = 0;
-        for (int p0 = 0; p0 < C;) {
-            // centre the frame on the furthest channel whose delays differ from those of
-            // p0 by amounts within 8 samples of each other, with moves of at most 16
-            const int32_t *d0 = dl.data() + (size_t)p0 * kKdm;
-            int best = p0;
-            for (int pos = p0; pos < C; pos++) {
-                const int32_t *d = dl.data() + (size_t)pos * kKdm;
-                const Range dv = range_of(d, d0), ev = range_of(d, R);
-                if (dv.hi - dv.lo > kMaxShift || (!first && ev.hi - ev.lo > kMaxMove)) break;
-                best = pos;
-            }
-            const int32_t *ref = dl.data() + (size_t)best * kKdm;
-            for (bool more = true; more;) {
-                const int elo = range_of(ref, R).lo;
-                MmaFrame fr;
-                fr.pos = p0;
-                more = false;
-                rmax = 0;
-                for (int i = 0; i < kKdm; i++) {
-                    int e = ref[i] - R[i] - elo;
-                    if (!first && e > kMaxMove) {  // a steep step: several moves
-                        e = kMaxMove;
-                        more = true;
-                    }
-                    fr.e[i] = first ? 0 : (uint8_t)e;
-                    R[i] += e;
-                    rmax = std::max(rmax, (int)R[i]);
-                }
-                fr.rmax = rmax;
-                if (rmax > 8 * kCols) return false;
-                t->frames.push_back(fr);
-                first = false;
-            }
-            int pos = p0;
-            for (; pos < C; pos++) {
-                const int32_t *d = dl.data() + (size_t)pos * kKdm;
-                const Range v = range_of(d, R);
-                if (v.hi - v.lo > kMaxShift) break;
-                t->base[(size_t)b * C + pos] = v.lo;
-                uint8_t *s = t->shift.data() + ((size_t)b * nchunk + pos / kChunk) * kKdm * kChunk + pos % kChunk;
-                for (int i = 0; i < kKdm; i++) s[i * kChunk] = (uint8_t)(d[i] - R[i] - v.lo);
-                int32_t &cr = t->crmax[(size_t)b * nchunk + pos / kChunk];
-                cr = std::max(cr, rmax);
-                t->mean_cols_r += rmax;
-            }
-            p0 = pos;
-        }
-        for (int i = 0; i < kKdm; i++) t->rlast[(size_t)b * kKdm + i] = R[i];
-        t->rmax = std::max(t->rmax, rmax);
         t->foff.push_back((int32_t)t->frames.size());
     }
-    t->mean_cols_r /= (double)nblk * C;
+    t->mean_cols_r /= (double)nblk * npos;
     return true;
+}
+
+int mma_split(const int32_t *delays, int ndm, int C, bool rev, int step, double other_rate) {
+    const int nblk = (ndm + kKdm - 1) / kKdm;
+    // the last block but one (complete, and as steep as any on a uniform grid)
+    std::vector<int32_t> dl((size_t)C * kKdm);
+    block_delays(delays, ndm, C, rev, C, std::max(0, nblk - 2), dl.data());
+    std::vector<MmaFrame> frames;
+    int32_t R[kKdm];
+    int reach = 0;  // positions whose rows stay within a tile
+    (void)block_frames(dl.data(), C, R, &frames, [&](int pos, int, int) { reach = pos + 1; });
+    double best = 0.9 * 16.0 * C / other_rate;  // clocks per sample of 16 trials: at least a tenth less
+    int npos = 0;
+    size_t f = 0;
+    double sum_r = 0.0;
+    int at = 0;
+    for (int rest = (C - 1) / step * step; rest > 0; rest -= step) {
+        const int n = C - rest;
+        if (n > reach) break;
+        for (; at < n; at++) {
+            while (f < frames.size() && frames[f].pos <= at) f++;
+            sum_r += frames[f - 1].rmax;
+        }
+        MmaShape m;
+        m.rmax = frames[f - 1].rmax + frames[f - 1].rmax / 8;  // other blocks may drift a little further
+        m.mean_r = sum_r / n;
+        m.frames_per_block = (double)f;
+        const int T = mma_tile_len(m.rmax);
+        if (T < 512 || n < 256) continue;
+        const double c = mma_item_clocks(m, n, T) / T + 16.0 * rest / other_rate;
+        if (c < best) {
+            best = c;
+            npos = n;
+        }
+    }
+    return npos;
 }
 
 int mma_tile_len(int rmax) { return std::max(0, (8 * kCols - rmax) & ~15); }
@@ -770,22 +844,25 @@ double mma_launch_clocks(const MmaShape &m, int nchan, int ndm, int64_t n_out, i
     return best;
 }
 
-cudaError_t launch_dedisperse_mma(const BeamLaunch *beams, int nbeams, int num_sms, int *err,
+cudaError_t launch_dedisperse_mma(const BeamLaunch *beams, int nbeams, bool add, int num_sms, int *err,
                                   cudaStream_t s, int32_t *nlaunch) {
     if (nbeams < 1 || nbeams > kMmaMaxBeams) return cudaErrorInvalidValue;
     cudaError_t e = ensure_kernel_smem(reinterpret_cast<const void *>(dd_mma_kernel), kSmem);
     if (e != cudaSuccess) return e;
     MmaArgs a;
     std::memset(&a, 0, sizeof(a));
-    a.nchan = beams[0].plan->desc.nchan;
+    a.nchan = beams[0].plan->mma.shape.npos;
     int64_t items = 0;
     for (int b = 0; b < nbeams; b++) {
         const BeamLaunch &in = beams[b];
         const gsp_plan_s *p = in.plan;
-        if (p->desc.nchan != a.nchan || !p->mma.d_frames) return cudaErrorInvalidValue;
+        if (p->mma.shape.npos != a.nchan || !p->mma.d_frames) return cudaErrorInvalidValue;
         MmaBeam &bt = a.beam[b];
-        bt.x = in.x;
+        bt.rev = p->desc.freq_descending ? 0 : 1;
+        // the first npos positions: the last npos rows, or the first ones
+        bt.x = in.x + (bt.rev ? (int64_t)(p->desc.nchan - a.nchan) * in.x_stride : 0);
         bt.x_stride = in.x_stride;
+        bt.add = add ? 1 : 0;
         bt.n_in = in.n_in;
         bt.n_out = in.n_out;
         bt.base = p->mma.d_base;
@@ -803,7 +880,6 @@ cudaError_t launch_dedisperse_mma(const BeamLaunch *beams, int nbeams, int num_s
         bt.ndm = p->desc.ndm;
         bt.nblk = (p->desc.ndm + kKdm - 1) / kKdm;
         bt.grp = p->geom.grp[kdm_index(kKdm)];
-        bt.rev = p->desc.freq_descending ? 0 : 1;
         if (in.bsum && bt.B < kMmaMinBlock) return cudaErrorInvalidValue;
         // the longest tiles for a batch, those of the best wave count for one beam
         const int tmax = mma_tile_len(p->mma.shape.rmax);

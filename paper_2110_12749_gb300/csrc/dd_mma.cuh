@@ -19,9 +19,9 @@ struct MmaFrame {
 };
 
 struct MmaTables {
-    std::vector<int32_t> base;     // [nblk][C] window start of each position, relative to the tile
-    std::vector<uint8_t> shift;    // [nblk][ceil(C / 8)][16][8] shift of each (position, DM), 0..8
-    std::vector<int32_t> crmax;    // [nblk][ceil(C / 8)] largest R of the chunk's frames
+    std::vector<int32_t> base;     // [nblk][npos] window start of each position, relative to the tile
+    std::vector<uint8_t> shift;    // [nblk][ceil(npos / 8)][16][8] shift of each (position, DM), 0..8
+    std::vector<int32_t> crmax;    // [nblk][ceil(npos / 8)] largest R of the chunk's frames
     std::vector<int32_t> rlast;    // [nblk][16] R of the last frame
     std::vector<int32_t> foff;     // [nblk + 1] first frame of each block
     std::vector<MmaFrame> frames;
@@ -31,14 +31,18 @@ struct MmaTables {
 
 // What the launch and the choice of kernel need of the tables.
 struct MmaShape {
+    int npos = 0;  // channels, in order of increasing delay
     int rmax = 0;
     double mean_r = 0.0;
     double frames_per_block = 0.0;
 };
 
-// delays [ndm][C]; rev: positions run from the last channel to the first.
-// false: a block's delays drift apart by more than a tile.
-bool mma_plan_tables(const int32_t *delays, int ndm, int C, bool rev, MmaTables *t);
+// delays [ndm][C]; rev: positions run from the last channel to the first; the first
+// npos of them.  false: a block's delays drift apart by more than a tile.
+bool mma_plan_tables(const int32_t *delays, int ndm, int C, bool rev, int npos, MmaTables *t);
+// How many positions to take where the rest (a multiple of step channels) is left to a
+// kernel of other_rate additions per clock and SM; 0 if that gains less than a tenth.
+int mma_split(const int32_t *delays, int ndm, int C, bool rev, int step, double other_rate);
 // Longest tile (output samples) for a largest R.
 int mma_tile_len(int rmax);
 // Estimated SM clocks of one work item (16 DM trials x T samples x nchan channels).

@@ -129,6 +129,7 @@ struct TiledArgs {
     int *err;      // set to 1 if a bounded wait gave up
     int64_t items;
     long long budget;  // SM clock cycles a pipeline wait may take before it gives up
+    int st0, st1;      // stages of channels to sum (all of them, or the steep ones)
     int starve;        // failure-path test: the producer issues nothing, so every stage wait
                        // runs out (no copy is ever in flight)
 };
@@ -370,7 +371,7 @@ __global__ void __launch_bounds__((KDM / KW + 1) * 32, (KDM / KW + 1) * 32 <= 25
         const BeamTile &bt = a.beam[bi];
         const int64_t t0 = tile * kTEff;
         const int32_t *bmin = bt.blkmin + (int64_t)blk * a.nchan;
-        for (int st = 0; st < nst && ok; st++, gst++) {
+        for (int st = a.st0; st < a.st1 && ok; st++, gst++) {
             if (wrapped) {
                 const bool w = ptx::mbar_wait(empty(slot), rpar ^ 1u, a.budget);
                 if (!__all_sync(0xffffffffu, w)) {
@@ -479,10 +480,10 @@ __global__ void __launch_bounds__((KDM / KW + 1) * 32, (KDM / KW + 1) * 32 <= 25
     const int32_t *dtab = PRE ? bt.dpos : bt.delays;
     const uint32_t *fcrow = PRE ? bt.fcnt + (int64_t)min(dmw, bt.ndm - 1) * nst : nullptr;
     int nx_min[kH], nx_dl[kKW][kH];
-    uint32_t nx_fc = PRE ? fcrow[0] : 0u;
+    uint32_t nx_fc = PRE ? fcrow[a.st0] : 0u;
 #pragma unroll
     for (int h = 0; h < kH; h++) {
-        const int c0 = h * 32 + lane;
+        const int c0 = a.st0 * kCB + h * 32 + lane;
         const bool v0 = c0 < a.nchan;
         nx_min[h] = v0 ? bmin[c0] : 0;
 #pragma unroll
@@ -490,12 +491,12 @@ __global__ void __launch_bounds__((KDM / KW + 1) * 32, (KDM / KW + 1) * 32 <= 25
             nx_dl[i][h] = v0 ? dtab[(int64_t)min(dmw + i, bt.ndm - 1) * a.nchan + c0] : 0;
     }
 
-    for (int st = 0; st < nst; st++) {
+    for (int st = a.st0; st < a.st1; st++) {
         int cur_min[kH], cur_dl[kKW][kH];
         // the same word in every lane; a warp reduction makes that visible to the compiler,
         // so the family loops below branch on a warp-uniform count
         const uint32_t cur_fc = PRE ? __reduce_or_sync(0xffffffffu, nx_fc) : 0u;
-        if (PRE && st + 1 < nst) nx_fc = fcrow[st + 1];
+        if (PRE && st + 1 < a.st1) nx_fc = fcrow[st + 1];
 #pragma unroll
         for (int h = 0; h < kH; h++) {
             cur_min[h] = nx_min[h];
@@ -675,10 +676,10 @@ __global__ void __launch_bounds__((KDM / KW + 1) * 32, (KDM / KW + 1) * 32 <= 25
             rpar ^= 1u;
         }
 
-        if (MF && ((st + 1) % kFlushStages == 0 || st == nst - 1)) {
+        if (MF && ((st + 1) % kFlushStages == 0 || st == a.st1 - 1)) {
 #pragma unroll
             for (int i = 0; i < kKW; i++) flush_merged<kM>(E[i], O[i], acc[i], lane);
-        } else if (FF && st == nst - 1) {
+        } else if (FF && st == a.st1 - 1) {
 #pragma unroll
             for (int i = 0; i < kKW; i++) {
                 flush_family<0, kM, ACC>(E[i][0], O[i][0], acc[i], lane);
@@ -686,7 +687,7 @@ __global__ void __launch_bounds__((KDM / KW + 1) * 32, (KDM / KW + 1) * 32 <= 25
                 flush_family<2, kM, ACC>(E[i][2], O[i][2], acc[i], lane);
                 flush_family<3, kM, ACC>(E[i][3], O[i][3], acc[i], lane);
             }
-        } else if (!MF && !FF && ((st + 1) % kFlushStages == 0 || st == nst - 1)) {
+        } else if (!MF && !FF && ((st + 1) % kFlushStages == 0 || st == a.st1 - 1)) {
 #pragma unroll
             for (int i = 0; i < kKW; i++) {
                 uint32_t sp[kM][3];
@@ -1063,12 +1064,22 @@ bool plan_dedisperse_tiled(gsp_plan_s *p, TiledTables *tab) {
     // clock and SM against 86; step 1.5 or a 500-3300 MHz band, whose delays drift
     // apart too fast: byte kernel).  A plan keeps its tables only if they may be used.
     int byte_variant = -1;
-    if (C <= kMmaMaxChannels && mma_plan_tables(p->delays_h.data(), ndm, C,
-                                                !p->desc.freq_descending, &tab->mma)) {
+    const bool rev = !p->desc.freq_descending;
+    bool split = false;
+    auto tables = [&](int npos) {
+        if (C > kMmaMaxChannels || !mma_plan_tables(p->delays_h.data(), ndm, C, rev, npos, &tab->mma)) {
+            tab->mma = MmaTables();
+            return false;
+        }
         MmaShape &m = p->mma.shape;
+        m.npos = npos;
         m.rmax = tab->mma.rmax;
         m.mean_r = tab->mma.mean_cols_r;
         m.frames_per_block = (double)tab->mma.frames.size() / (double)((ndm + 15) / 16);
+        return true;
+    };
+    if (tables(C)) {
+        MmaShape &m = p->mma.shape;
         const int T = mma_tile_len(m.rmax);
         const double byte_clk = 16.0 * T * C / byte_rate(variant);
         const double mma_clk = T >= kMmaMinTile ? mma_item_clocks(m, C, T) : 1e30;
@@ -1080,11 +1091,20 @@ bool plan_dedisperse_tiled(gsp_plan_s *p, TiledTables *tab) {
             byte_variant = variant;
             variant = kMmaVariant;
         }
-    } else {
-        tab->mma = MmaTables();
+    }
+    // A band of which only a part drifts slowly enough: the tensor-core kernel for that
+    // part, the byte kernel for the whole stages of steep channels before it (2048
+    // channels, 500-3300 MHz, 3000 trials, 600011 samples: 26.7 -> 22.2 ms).
+    if (!forced && !force_mma && variant != kMmaVariant) {
+        const int npos = mma_split(p->delays_h.data(), ndm, C, rev, 64, byte_rate(variant));
+        if (npos > 0) {
+            split = tables(npos) && mma_tile_len(p->mma.shape.rmax) >= kMmaMinTile;
+            if (!split) tab->mma = MmaTables();
+        }
     }
     dedisperse_set_variant(p, variant);
     g.byte_variant = byte_variant;
+    g.split = split;
     return true;
 }
 
@@ -1103,7 +1123,7 @@ TileFit dedisperse_fit(int variant, const int64_t (&spread)[kNumKdm]) {
 
 bool dedisperse_variant_usable(const gsp_plan_s *p, int variant) {
     if (!p || p->simple_dd || variant < 0 || variant > kMmaVariant) return false;
-    if (variant == kMmaVariant) return p->mma.d_frames != nullptr;
+    if (variant == kMmaVariant) return p->mma.d_frames != nullptr && p->mma.shape.npos == p->desc.nchan;
     const TiledVariant &v = kVariants[variant];
     const int o = kdm_index(v.kdm), ci = cb_index(v.cb);
     if (!p->d_blkmin[o] || !p->d_stspread[o][ci]) return false;
@@ -1122,6 +1142,7 @@ void dedisperse_set_variant(gsp_plan_s *p, int variant) {
         g.ctas_per_sm = 1;
         g.variant = variant;
         g.byte_variant = -1;
+        g.split = false;
         return;
     }
     const TiledVariant &v = kVariants[variant];
@@ -1137,6 +1158,7 @@ void dedisperse_set_variant(gsp_plan_s *p, int variant) {
     g.ctas_per_sm = f.ctas_per_sm;
     g.variant = variant;
     g.byte_variant = -1;
+    g.split = false;
 }
 
 int dedisperse_choose_variant(const gsp_plan_s *const *plans, int nplans) {
@@ -1152,29 +1174,18 @@ int dedisperse_choose_variant(const gsp_plan_s *const *plans, int nplans) {
     const int v0 = plans[0]->geom.variant;
     bool same = true;
     for (int i = 1; i < nplans; i++) same = same && plans[i]->geom.variant == v0;
-    if (same && v0 == kMmaVariant) return v0;
+    if (same && v0 == kMmaVariant) return v0;  // every plan keeps its tables for all channels
     if (same && v0 < kNumVariants && lists_ok(kVariants[v0], have_lists[cb_index(kVariants[v0].cb)]) &&
         fit_variant(kVariants[v0], spread[kdm_index(kVariants[v0].kdm)]).ok)
         return v0;
     return choose_auto(spread, have_lists);
 }
 
-cudaError_t launch_dedisperse_batch(const BeamLaunch *beams, int nbeams, int variant,
-                                    bool persistent, int num_sms, int *err, cudaStream_t s,
-                                    int32_t *nlaunch) {
-    if (nbeams < 1 || nbeams > kMaxBatchBeams || variant < 0 || variant > kMmaVariant)
-        return cudaErrorInvalidValue;
-    if (variant == kMmaVariant) {
-        // one short beam: the byte kernel where its waves are estimated to end earlier
-        const gsp_plan_s *p = beams[0].plan;
-        const int bv = p->geom.byte_variant;
-        int T = 0;
-        if (nbeams > 1 || bv < 0 ||
-            mma_launch_clocks(p->mma.shape, p->desc.nchan, p->desc.ndm, beams[0].n_out, num_sms, &T) <=
-                byte_launch_clocks(bv, p->desc.nchan, p->desc.ndm, beams[0].n_out, num_sms))
-            return launch_dedisperse_mma(beams, nbeams, num_sms, err, s, nlaunch);
-        variant = bv;
-    }
+namespace {
+
+// The byte kernel on the channels [c0, c1) of every beam (c0 a whole stage).
+cudaError_t launch_bytes(const BeamLaunch *beams, int nbeams, int variant, bool persistent, int c0, int c1,
+                         int num_sms, int *err, cudaStream_t s, int32_t *nlaunch) {
     const TiledVariant &v = kVariants[variant];
     const int o = kdm_index(v.kdm), ci = cb_index(v.cb);
     const int t_cta = 128 * v.m, t_eff = t_cta - 4;
@@ -1230,6 +1241,8 @@ cudaError_t launch_dedisperse_batch(const BeamLaunch *beams, int nbeams, int var
     a.one = 1u;
     a.err = err;
     a.items = items;
+    a.st0 = c0 / v.cb;
+    a.st1 = (c1 + v.cb - 1) / v.cb;
     a.budget = beams[0].plan->wait_budget;
     a.starve = beams[0].plan->wait_starve;
     int64_t grid = persistent ? std::min<int64_t>(items, (int64_t)num_sms * f.ctas_per_sm) : items;
@@ -1237,6 +1250,44 @@ cudaError_t launch_dedisperse_batch(const BeamLaunch *beams, int nbeams, int var
     v.fn<<<(unsigned)grid, (v.kdm / v.kw + 1) * 32, f.smem, s>>>(a);
     *nlaunch += 1;
     return cudaGetLastError();
+}
+
+}  // namespace
+
+cudaError_t launch_dedisperse_batch(const BeamLaunch *beams, int nbeams, int variant, bool persistent,
+                                    int num_sms, int *err, cudaStream_t s, int32_t *nlaunch) {
+    if (nbeams < 1 || nbeams > kMaxBatchBeams || variant < 0 || variant > kMmaVariant)
+        return cudaErrorInvalidValue;
+    const gsp_plan_s *p = beams[0].plan;
+    const int C = p->desc.nchan, ndm = p->desc.ndm;
+    const int64_t n_out = beams[0].n_out;
+    int T = 0;
+    if (variant == kMmaVariant) {
+        // one short beam: the byte kernel where its waves are estimated to end earlier
+        const int bv = p->geom.byte_variant;
+        if (nbeams > 1 || bv < 0 ||
+            mma_launch_clocks(p->mma.shape, C, ndm, n_out, num_sms, &T) <=
+                byte_launch_clocks(bv, C, ndm, n_out, num_sms))
+            return launch_dedisperse_mma(beams, nbeams, false, num_sms, err, s, nlaunch);
+        variant = bv;
+    } else if (nbeams == 1 && p->geom.split && variant == p->geom.variant &&
+               (!beams[0].bsum || p->desc.block_len >= kMmaMinBlock)) {
+        // the steep channels' sums first, then the others' added to them
+        const int n1 = p->mma.shape.npos;
+        if (mma_launch_clocks(p->mma.shape, n1, ndm, n_out, num_sms, &T) +
+                byte_launch_clocks(variant, C - n1, ndm, n_out, num_sms) <
+            byte_launch_clocks(variant, C, ndm, n_out, num_sms)) {
+            BeamLaunch steep = beams[0];
+            steep.bsum = nullptr;
+            const int c0 = p->desc.freq_descending ? n1 : 0, c1 = p->desc.freq_descending ? C : C - n1;
+            if (c0 % kVariants[variant].cb == 0 && (c1 == C || c1 % kVariants[variant].cb == 0)) {
+                cudaError_t e = launch_bytes(&steep, 1, variant, persistent, c0, c1, num_sms, err, s, nlaunch);
+                if (e != cudaSuccess) return e;
+                return launch_dedisperse_mma(beams, 1, true, num_sms, err, s, nlaunch);
+            }
+        }
+    }
+    return launch_bytes(beams, nbeams, variant, persistent, 0, C, num_sms, err, s, nlaunch);
 }
 
 cudaError_t launch_dedisperse_tiled(const gsp_plan_s *p, const uint8_t *x, int64_t n_in,

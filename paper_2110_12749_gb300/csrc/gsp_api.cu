@@ -763,11 +763,15 @@ gsp_status gsp_plan_tune(gsp_plan_t p, const uint8_t *d_x, int64_t n_in, int64_t
     const int *cand = nullptr;
     const int ncand = gsp::dedisperse_tune_candidates(&cand);
     const int keep = p->geom.variant;
+    const bool split = p->geom.split;  // the plan's split between two kernels is timed too
     int best = -1;
+    bool best_split = false;
     float best_t = 0.f;
-    for (int ci = 0; ci < ncand; ci++) {
-        if (!gsp::dedisperse_variant_usable(p, cand[ci])) continue;
-        gsp::dedisperse_set_variant(p, cand[ci]);
+    for (int ci = 0; ci < ncand + (split ? 1 : 0); ci++) {
+        const int v = ci < ncand ? cand[ci] : keep;
+        if (!gsp::dedisperse_variant_usable(p, v)) continue;
+        gsp::dedisperse_set_variant(p, v);
+        p->geom.split = ci == ncand;
         std::vector<float> ms;
         for (int r = 0; r <= kPlanTuneReps; r++) {
             int32_t nl = 0;
@@ -776,6 +780,7 @@ gsp_status gsp_plan_tune(gsp_plan_t p, const uint8_t *d_x, int64_t n_in, int64_t
                                                          p->d_D, stride, nullptr, s, &nl);
             if (e != cudaSuccess) {
                 gsp::dedisperse_set_variant(p, keep);
+                p->geom.split = split;
                 set_err(e, "tuning launch");
                 return GSP_ERR_CUDA;
             }
@@ -788,12 +793,14 @@ gsp_status gsp_plan_tune(gsp_plan_t p, const uint8_t *d_x, int64_t n_in, int64_t
         std::sort(ms.begin(), ms.end());
         const float med = ms[ms.size() / 2];
         if (best < 0 || med < best_t) {
-            best = cand[ci];
+            best = v;
+            best_split = ci == ncand;
             best_t = med;
         }
     }
     gsp_status kst = take_kernel_error(p);
     gsp::dedisperse_set_variant(p, best >= 0 ? best : keep);
+    p->geom.split = best >= 0 ? best_split : split;
     if (kst != GSP_OK) return kst;
     if (variant) *variant = p->geom.variant;
     if (best_ms) *best_ms = best_t;

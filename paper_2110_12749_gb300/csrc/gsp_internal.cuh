@@ -62,6 +62,9 @@ struct DDGeom {
     // the plan's choice by estimate was the tensor-core kernel: a launch takes this byte
     // variant instead where it is estimated the faster (-1: the variant is fixed)
     int byte_variant = -1;
+    // the plan's choice was a byte variant for the steep channels and the tensor-core kernel
+    // for the first mma.shape.npos positions (launches of one beam)
+    bool split = false;
 };
 
 // Launch geometry of one tile variant for a given largest in-block delay
@@ -184,7 +187,8 @@ cudaError_t launch_dedisperse_batch(const BeamLaunch *beams, int nbeams, int var
                                     bool persistent, int num_sms, int *err, cudaStream_t s,
                                     int32_t *nlaunch);
 // The same on the tensor cores (plans that keep the MmaDevice tables).
-cudaError_t launch_dedisperse_mma(const BeamLaunch *beams, int nbeams, int num_sms, int *err,
+// add: to the series that is there.
+cudaError_t launch_dedisperse_mma(const BeamLaunch *beams, int nbeams, bool add, int num_sms, int *err,
                                   cudaStream_t s, int32_t *nlaunch);
 int dedisperse_num_variants();
 // Variants the batch autotuner may time, in order of preference.
