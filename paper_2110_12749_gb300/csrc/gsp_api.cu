@@ -597,7 +597,7 @@ gsp_status gsp_candidates(gsp_plan_t p, gsp_cand *host_out, int64_t cap, int64_t
 // aligned and its block sums land in whole blocks; chunk k needs the input
 // columns [a_k, a_{k+1} + max_delay), and its copy brings the columns not yet
 // on the device.  The series are exact integer sums, so the result does not
-// depend on the chunking.  GSP_HOST_CHUNKS (1..8) sets the number of chunks;
+// depend on the chunking.  At most 8 chunks; GSP_HOST_CHUNKS (1..8) sets the number,
 // 1 copies everything first.
 constexpr int kHostChunks = 8;
 
@@ -607,6 +607,14 @@ int host_chunks() {
         if (k >= 1 && k <= kHostChunks) return k;
     }
     return kHostChunks;
+}
+
+// Relative size of chunk k of n: 1, 1, 2, 4, 8, 8, 8, 8; and their sum.
+static int64_t chunk_weight(int k) { return k == 0 ? 1 : std::min<int64_t>((int64_t)1 << (k - 1), 8); }
+static int64_t chunk_weights(int n) {
+    int64_t sum = 0;
+    for (int k = 0; k < n; k++) sum += chunk_weight(k);
+    return sum;
 }
 
 gsp_status gsp_search_host(gsp_plan_t p, const uint8_t *h_x, int64_t n_in, int64_t x_stride,
@@ -631,7 +639,14 @@ gsp_status gsp_search_host(gsp_plan_t p, const uint8_t *h_x, int64_t n_in, int64
     const int64_t B = p->desc.block_len;
     int64_t unit = B;
     while (unit % 16) unit += B;  // lcm(B, 16)
-    const int nch = host_chunks();
+    // fewer chunks for a short series: the smallest one should fill four waves of the
+    // dedispersion kernel's work items (131072 samples in 8 chunks: 20.5 ms of launches
+    // whose last waves are part empty, against 16.1 ms in one)
+    int nch = host_chunks();
+    if (!std::getenv("GSP_HOST_CHUNKS")) {
+        const int64_t fill = 4 * (int64_t)p->num_sms * p->geom.t_cta * p->geom.kdm / std::max(p->desc.ndm, 1);
+        while (nch > 3 && n_out < chunk_weights(nch) * fill) nch--;
+    }
     const bool pipelined = nch > 1 && !p->simple_dd && n_out >= nch * unit;
     if (!pipelined) {
         if (x_stride == dstride) {
@@ -651,16 +666,12 @@ gsp_status gsp_search_host(gsp_plan_t p, const uint8_t *h_x, int64_t n_in, int64
     // launch waits only for a small copy (its columns plus the max_delay
     // overhang), and each later copy is at most the size of the launch it hides
     // behind; equal chunks when the series is too short for the smallest ones
-    int64_t wts[kHostChunks], wsum = 0;
-    for (int k = 0; k < nch; k++) {
-        wts[k] = k == 0 ? 1 : std::min<int64_t>((int64_t)1 << (k - 1), 8);
-        wsum += wts[k];
-    }
+    const int64_t wsum = chunk_weights(nch);
     const bool grow = n_out >= wsum * unit;
     int64_t a[kHostChunks + 1];
     a[0] = 0;
     for (int k = 0, cum = 0; k < nch; k++) {
-        cum += (int)wts[k];
+        cum += (int)chunk_weight(k);
         a[k + 1] = (grow ? n_out * cum / wsum : n_out * (k + 1) / nch) / unit * unit;
     }
     a[nch] = n_out;
