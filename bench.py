@@ -27,14 +27,13 @@ ROOT = os.path.dirname(os.path.abspath(__file__))
 if ROOT not in sys.path:
     sys.path.insert(0, ROOT)
 
-# DRAM bytes (read + write) per algorithmic add of the default dedispersion kernel
-# (variant 32, with per-stage copy windows and warp-uniform family counts): ncu
+# DRAM bytes (read + write) per algorithmic add of the byte kernel (variant 32): ncu
 # dram__bytes_read.sum + dram__bytes_write.sum of one launch on the CRAFTS-like beam
 # cut to 131072 samples (1.574 GB + 0.665 GB for 6.899e11 adds), the capture size
 # rule keeping full-size multi-pass captures off the GPU; traffic grows with the
 # number of time tiles, i.e. in proportion to the adds.
 DD_TRAFFIC_BYTES_PER_ADD = (1.5738e9 + 0.6653e9) / 6.899e11
-DD_TRAFFIC_VARIANT = "default"
+DD_TRAFFIC_VARIANT = 32
 
 NOMINAL_SMS = 152
 RANKER_KEYS = ("recall", "recall_nominal", "precision", "precision_snr8", "negatives_rejected", "threshold",
@@ -43,7 +42,16 @@ RANKER_KEYS = ("recall", "recall_nominal", "precision", "precision_snr8", "negat
                "train_snippets", "train_positives", "train_steps", "train_steps_per_s", "params",
                "recipe")
 INT_LANES_PER_SM = 128          # issue slots per SM per clock (4 schedulers x 32 lanes)
+TENSOR_ADDS_PER_SM = 256        # additions per SM per clock of the tensor-core kernel: a K = 16
+                                # product (16 multiply-adds of 4096 per clock) does one
+TENSOR_VARIANT = 45             # index of that kernel among the dedispersion variants
 SM_MAX_MHZ = 2070.0
+
+
+def dd_peak(nsm, variant):
+    """Peak of a dedispersion variant in T additions per second (maximum SM clock)."""
+    per_sm = TENSOR_ADDS_PER_SM if variant == TENSOR_VARIANT else INT_LANES_PER_SM
+    return nsm * per_sm * SM_MAX_MHZ * 1e6 / 1e12
 
 
 def parse():
@@ -465,7 +473,7 @@ def run_batch(args, wl):
     torch.cuda.empty_cache()
     ms_dd, ms_tot = float(np.median(dd)), float(np.median(tot))
     nsm = torch.cuda.get_device_properties(torch.cuda.current_device()).multi_processor_count
-    peak = nsm * INT_LANES_PER_SM * SM_MAX_MHZ * 1e6 / 1e12
+    peak = dd_peak(nsm, variant)
     return {"beams": B, "samples_total": int(sum(n_ins)), "sky_s": _r(sky), "adds": _r(adds),
             "ms_per_batch": _r(ms_tot), "dedisperse_ms": _r(ms_dd),
             "sky_s_per_s": _r(sky / (ms_tot / 1e3)),
@@ -518,7 +526,7 @@ def run_wideband(args):
     adds = float(wl.ndm) * wl.nchan * n_out
     ms_dd, ms_tot = float(np.median(dd)), float(np.median(tot))
     nsm = torch.cuda.get_device_properties(torch.cuda.current_device()).multi_processor_count
-    peak = nsm * INT_LANES_PER_SM * SM_MAX_MHZ * 1e6 / 1e12
+    peak = dd_peak(nsm, variant)
     return {"workload": workload_desc(wl), "n_out": n_out, "max_delay": wl.n_in - n_out,
             "variant_auto": auto, "variant": variant, "ms_per_step": _r(ms_tot),
             "dedisperse_ms": _r(ms_dd), "search_ms": _r(float(np.median(se))),
@@ -828,7 +836,9 @@ def run_gsp(args):
     achieved = adds / (dd_avg / 1e3) / 1e12            # T adds / s
     nsm = torch.cuda.get_device_properties(local).multi_processor_count
     clocks = clk.summary()
-    peak = nsm * INT_LANES_PER_SM * SM_MAX_MHZ * 1e6 / 1e12
+    dd_used = gsp.gsp_dedisperse_variants(plan)[1]
+    dd_tensor = dd_used == TENSOR_VARIANT
+    peak = dd_peak(nsm, dd_used)
     line = None
     stream_res = None
     batch_res = None
@@ -873,14 +883,13 @@ def run_gsp(args):
             "config": bench_config(wl, n_out, world),
             "dm_chan_samples_per_s": world * adds / (ms_step / 1e3),
             "kernel_ms": {"dedisperse": dd_avg, "search": sum(se_ms) / len(se_ms)},
-            "roofline": {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "Tadd/s",
+            "roofline": {"bound": "tensor" if dd_tensor else "alu", "achieved": achieved, "peak": peak, "unit": "Tadd/s",
                          "frac": achieved / peak,
-                         "traffic": (DD_TRAFFIC_BYTES_PER_ADD * adds
-                                     if os.environ.get("GSP_DD_VARIANT", "default") == DD_TRAFFIC_VARIANT
-                                     else None),
-                         "peak_basis": "%d SMs x %d int lanes x %.0f MHz (max clock)"
-                                       % (nsm, INT_LANES_PER_SM, SM_MAX_MHZ),
-                         "frac_at_run_clock": (achieved / (nsm * INT_LANES_PER_SM * clocks["sm_mhz"] * 1e-6)
+                         "traffic": (DD_TRAFFIC_BYTES_PER_ADD * adds if dd_used == DD_TRAFFIC_VARIANT else None),
+                         "peak_basis": "%d SMs x %d %s x %.0f MHz (max clock)"
+                                       % (nsm, TENSOR_ADDS_PER_SM if dd_tensor else INT_LANES_PER_SM,
+                                          "adds of a K = 16 product" if dd_tensor else "int lanes", SM_MAX_MHZ),
+                         "frac_at_run_clock": (achieved / (peak * clocks["sm_mhz"] / SM_MAX_MHZ)
                                                if clocks["sm_mhz"] else None)},
             "e2e": {"value": e2e_value, "unit": "sky-s/s", "ms_per_step": e2e_step,
                     "h2d_bytes_per_step": h2d, "d2h_bytes_per_step": 8 + 24 * int(n2),
