@@ -203,8 +203,9 @@ gsp_status gsp_candidates(gsp_plan_t plan, gsp_cand *host_out, int64_t cap,
 /* End-to-end call on HOST data: copies h_x (host, pinned or pageable,
  * x_stride bytes per channel) to plan-owned device memory, runs gsp_search
  * and returns the candidates as gsp_candidates does.  Synchronises.  With the
- * tiled kernel the input is copied in time chunks (8 by default; environment
- * variable GSP_HOST_CHUNKS = 1..8, 1 = copy everything first) on a second
+ * tiled kernel the input is copied in time chunks (8 by default, fewer for a
+ * short series; environment variable GSP_HOST_CHUNKS = 1..8 sets the number, 1 =
+ * copy everything first) on a second
  * stream, each chunk's dedispersion starting when its columns have arrived,
  * so that the copy of chunk k + 1 overlaps the dedispersion of chunk k
  * (overlap needs pinned host memory).  The result does not depend on the
@@ -241,7 +242,8 @@ gsp_status gsp_plan_set_wait_limit(gsp_plan_t plan, int64_t cycles, int32_t star
  * the number of variants; if plan is not NULL and in_use is not NULL, writes
  * the variant the plan uses, or -1 if it uses the simple kernel.  A plan's
  * variant is chosen at gsp_plan_create: the index in the environment variable
- * GSP_DD_VARIANT if that is in range and fits the plan, else the first of a
+ * GSP_DD_VARIANT if that is in range and fits the plan, else the tensor-core
+ * kernel (the last index) where it is estimated to be faster, else the first of a
  * preference list (64-channel stages; 32-channel stages; 7-DM blocks) whose
  * shared-memory stages hold the plan's largest in-block delay spread with at
  * least two ring slots.  The simple kernel (-1) is used only with

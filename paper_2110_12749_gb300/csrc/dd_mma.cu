@@ -754,26 +754,36 @@ bool mma_plan_tables(const int32_t *delays, int ndm, int C, bool rev, int npos, 
     t->frames.clear();
     t->rmax = 0;
     t->mean_cols_r = 0.0;
-    std::vector<int32_t> dl((size_t)npos * kKdm);
-    for (int b = 0; b < nblk; b++) {
-        block_delays(delays, ndm, C, rev, npos, b, dl.data());
-        int32_t R[kKdm];
-        const bool ok = block_frames(dl.data(), npos, R, &t->frames, [&](int pos, int lo, int rmax) {
-            const int32_t *d = dl.data() + (size_t)pos * kKdm;
-            t->base[(size_t)b * npos + pos] = lo;
-            uint8_t *sh = t->shift.data() + ((size_t)b * nchunk + pos / kChunk) * kKdm * kChunk + pos % kChunk;
-            for (int i = 0; i < kKdm; i++) sh[i * kChunk] = (uint8_t)(d[i] - R[i] - lo);
-            int32_t &cr = t->crmax[(size_t)b * nchunk + pos / kChunk];
-            cr = std::max(cr, rmax);
-            t->mean_cols_r += rmax;
-        });
-        if (!ok) return false;
-        for (int i = 0; i < kKdm; i++) {
-            t->rlast[(size_t)b * kKdm + i] = R[i];
-            t->rmax = std::max(t->rmax, (int)R[i]);
+    // the blocks are independent; their frames are put together at the end
+    std::vector<std::vector<MmaFrame>> fr((size_t)nblk);
+    std::vector<double> sum_r((size_t)nblk, 0.0);
+    std::atomic<bool> fits{true};
+    const bool ran = parallel_ranges(nblk, std::max(1, 100000 / (npos * kKdm)), [&](int64_t b0, int64_t b1) {
+        std::vector<int32_t> dl((size_t)npos * kKdm);
+        for (int64_t b = b0; b < b1 && fits; b++) {
+            block_delays(delays, ndm, C, rev, npos, (int)b, dl.data());
+            int32_t R[kKdm];
+            if (!block_frames(dl.data(), npos, R, &fr[b], [&](int pos, int lo, int rmax) {
+                    const int32_t *d = dl.data() + (size_t)pos * kKdm;
+                    t->base[(size_t)b * npos + pos] = lo;
+                    uint8_t *sh = t->shift.data() + ((size_t)b * nchunk + pos / kChunk) * kKdm * kChunk +
+                                  pos % kChunk;
+                    for (int i = 0; i < kKdm; i++) sh[i * kChunk] = (uint8_t)(d[i] - R[i] - lo);
+                    int32_t &cr = t->crmax[(size_t)b * nchunk + pos / kChunk];
+                    cr = std::max(cr, rmax);
+                    sum_r[b] += rmax;
+                }))
+                fits = false;
+            for (int i = 0; i < kKdm; i++) t->rlast[(size_t)b * kKdm + i] = R[i];
         }
+    });
+    if (!ran || !fits) return false;
+    for (int b = 0; b < nblk; b++) {
+        t->frames.insert(t->frames.end(), fr[b].begin(), fr[b].end());
         t->foff.push_back((int32_t)t->frames.size());
+        t->mean_cols_r += sum_r[b];
     }
+    for (int32_t r : t->rlast) t->rmax = std::max(t->rmax, (int)r);
     t->mean_cols_r /= (double)nblk * npos;
     return true;
 }

@@ -1,7 +1,9 @@
 // Brute-force incoherent dedispersion kernels (Sec. 2.3, Alg. 2/3):
 //   D[dm][t] = sum_c X[c][t + delay[dm][c]],  t < n_out = n_in - max delay.
 //
-// The tiled kernel (dd_tiled_kernel) is the performance path.  Each CTA owns
+// Most plans run on the tensor cores (dd_mma.cu).  The tiled kernel of this file
+// (dd_tiled_kernel) takes what they cannot or what is too small for them: steep
+// channels, launches of few work items, plans outside their limits.  Each CTA owns
 // a tile of KW*8 consecutive DM trials x T_EFF output samples and streams the
 // channels through a ring of shared-memory stages (32 channels per stage).
 // A producer warp fills a stage with one TMA bulk copy per channel: the
@@ -961,17 +963,24 @@ void plan_phase_lists(const gsp_plan_s *p, int cb, std::vector<int32_t> *dpos,
     if (p->max_delay >= ((int64_t)1 << 23)) return;  // packed delay field is 23 bits
     dpos->resize((size_t)ndm * C);
     fcnt->resize((size_t)ndm * nst);
-    for (int d = 0; d < ndm; d++) {
-        const int32_t *dl = p->delays_h.data() + (size_t)d * C;
-        for (int st = 0; st < nst; st++) {
-            uint32_t cnt[4] = {0, 0, 0, 0};
-            for (int c = st * cb; c < std::min(C, st * cb + cb); c++) {
-                const int P = dl[c] & 3;
-                (*dpos)[(size_t)d * C + c] = (int32_t)(((uint32_t)dl[c] << 8) | (uint32_t)(P * cb + cnt[P]));
-                cnt[P]++;
+    const bool ran = parallel_ranges(ndm, std::max(1, 200000 / C), [&](int64_t d0, int64_t d1) {
+        for (int64_t d = d0; d < d1; d++) {
+            const int32_t *dl = p->delays_h.data() + (size_t)d * C;
+            int32_t *pos = dpos->data() + (size_t)d * C;
+            for (int st = 0; st < nst; st++) {
+                uint32_t cnt[4] = {0, 0, 0, 0};
+                for (int c = st * cb; c < std::min(C, st * cb + cb); c++) {
+                    const int P = dl[c] & 3;
+                    pos[c] = (int32_t)(((uint32_t)dl[c] << 8) | (uint32_t)(P * cb + cnt[P]));
+                    cnt[P]++;
+                }
+                (*fcnt)[(size_t)d * nst + st] = cnt[0] | (cnt[1] << 8) | (cnt[2] << 16) | (cnt[3] << 24);
             }
-            (*fcnt)[(size_t)d * nst + st] = cnt[0] | (cnt[1] << 8) | (cnt[2] << 16) | (cnt[3] << 24);
         }
+    });
+    if (!ran) {
+        dpos->clear();
+        fcnt->clear();
     }
 }
 

@@ -57,18 +57,30 @@ gsp_status compute_delays(const gsp_plan_desc *d, const std::vector<double> &dms
         const double f = d->f_lo_mhz + ((double)k + 0.5) * df;
         law[c] = 1.0 / (f * f) - inv_top2;
     }
-    for (size_t i = 0; i < dms.size(); i++) {
-        const double dm = dms[i];
-        for (int64_t c = 0; c < C; c++) {
-            const double x = 4.148808e3 * dm * law[c] / d->t_samp_s;
-            const double fl = std::floor(x);
-            const double m = std::fabs((x - fl) - 0.5);
-            if (m < margin) margin = m;
-            const double r = std::floor(x + 0.5);
-            if (!(r >= 0.0) || r > 2147483647.0) return GSP_ERR_INVALID_ARG;
-            out[i * C + c] = (int32_t)r;
+    std::vector<double> margins(dms.size(), 1.0);
+    std::atomic<bool> valid{true};
+    const bool ran = gsp::parallel_ranges((int64_t)dms.size(), std::max<int64_t>(1, 200000 / C), [&](int64_t i0, int64_t i1) {
+        for (int64_t i = i0; i < i1; i++) {
+            const double dm = dms[i];
+            double least = 1.0;
+            for (int64_t c = 0; c < C; c++) {
+                const double x = 4.148808e3 * dm * law[c] / d->t_samp_s;
+                const double fl = std::floor(x);
+                const double m = std::fabs((x - fl) - 0.5);
+                if (m < least) least = m;
+                const double r = std::floor(x + 0.5);
+                if (!(r >= 0.0) || r > 2147483647.0) {
+                    valid = false;
+                    return;
+                }
+                out[i * C + c] = (int32_t)r;
+            }
+            margins[i] = least;
         }
-    }
+    });
+    if (!ran) return GSP_ERR_OOM;
+    if (!valid) return GSP_ERR_INVALID_ARG;
+    for (double m : margins) margin = std::min(margin, m);
     if (min_margin) *min_margin = margin;
     return GSP_OK;
 }

@@ -3,7 +3,10 @@
 
 #include <cuda_runtime.h>
 
+#include <algorithm>
+#include <atomic>
 #include <cstdint>
+#include <thread>
 #include <vector>
 
 #include "dd_mma.cuh"
@@ -13,6 +16,33 @@ namespace gsp {
 
 constexpr int kMaxWidths = 32;
 constexpr long long kWaitLimit = 4000000000ll;  // ~2 s of SM clock: the longest bounded wait
+
+// fn(begin, end) over [0, n) on up to 8 host threads, each with at least `grain`
+// indices; on the calling thread alone for less.  false if a call threw (the
+// ranges are independent, so the caller may report or repeat it).
+template <typename Fn>
+bool parallel_ranges(int64_t n, int64_t grain, Fn fn) {
+    const int64_t hw = std::max(1u, std::thread::hardware_concurrency());
+    const int64_t nt = std::max<int64_t>(1, std::min<int64_t>(std::min<int64_t>(8, hw), n / std::max<int64_t>(grain, 1)));
+    std::atomic<bool> ok{true};
+    auto run = [&](int64_t i) {
+        try {
+            fn(n * i / nt, n * (i + 1) / nt);
+        } catch (...) {
+            ok = false;
+        }
+    };
+    std::thread pool[8];
+    int64_t started = 1;  // range 0 is this thread's
+    try {
+        for (; started < nt; started++) pool[started] = std::thread(run, started);
+    } catch (...) {
+    }
+    run(0);
+    for (int64_t i = started; i < nt; i++) run(i);  // those that got no thread
+    for (int64_t i = 1; i < started; i++) pool[i].join();
+    return ok;
+}
 
 // DM trials per CTA of the tiled dedispersion kernel (one per consumer warp):
 // 16; 15 so that the CTA (15 consumer warps + 1 producer) is 16 warps and each
