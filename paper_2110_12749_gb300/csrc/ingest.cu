@@ -1,22 +1,42 @@
 // Ingest transpose: time-major 8-bit samples [N][C] (the order of PSRFITS
 // files and of Alg. 2's numpts x numchan input matrix, Sec. 2.3) into the
 // channel-major [C][N] layout the dedispersion kernels read.  HBM-bound: one
-// read and one write per byte.  A CTA moves a 64 x 64 byte tile through shared
-// memory, with 16-byte global accesses when pointers and strides allow
-// (ingest_transpose16_kernel), else 4-byte or byte accesses.
+// read and one write per byte.  Rows of the output that are 16-byte aligned take
+// ingest_transpose16_kernel, whatever the input's alignment; others a kernel of
+// 64 x 64 byte tiles with 4-byte or byte accesses.
+//
+// A tile is 64 channels wide, half of a 128-byte line of the input.  Tiles are
+// therefore visited in groups of kGroup channel tiles side by side before the next
+// time tile: with all time tiles of one channel tile first, every line comes from
+// memory in two halves at different times (4096 x 2^20 samples, one / two / four /
+// eight / all side by side: 2076 / 1377 / 1368 / 1376 / 1377 us; rows of 2^20 + 16
+// bytes: 2151 / 1491 / 1490 / 1508 / 1548).
 #include "gsp_internal.cuh"
 
 namespace {
 
 constexpr int kTile = 64;
+constexpr unsigned kGroup = 4;
+
+// Tile of this CTA: grid (time tiles, channel tiles), renumbered within each kGroup
+// rows of the grid.  32 bits hold the number: more than 2^30 time tiles and more than
+// one channel tile would be over 2^42 bytes.
+__device__ __forceinline__ void tile_of(unsigned *tt, unsigned *ct) {
+    const unsigned c0 = blockIdx.y / kGroup * kGroup, g = min(kGroup, gridDim.y - c0);
+    const unsigned k = (blockIdx.y - c0) * gridDim.x + blockIdx.x;
+    *tt = k / g;
+    *ct = c0 + k % g;
+}
 
 __global__ void __launch_bounds__(256) ingest_transpose_kernel(const uint8_t *__restrict__ in,
                                                                int64_t in_stride, int64_t N, int C,
                                                                uint8_t *__restrict__ out,
                                                                int64_t out_stride, bool words) {
     __shared__ uint8_t tile[kTile][kTile + 4];
-    const int64_t t0 = (int64_t)blockIdx.x * kTile;   // time
-    const int c0 = blockIdx.y * kTile;                // channel
+    unsigned tt, ct;
+    tile_of(&tt, &ct);
+    const int64_t t0 = (int64_t)tt * kTile;   // time
+    const int c0 = (int)ct * kTile;           // channel
     const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;  // 16 x 16 threads
     // load: rows are times, 4 channels per thread
     for (int r = ty; r < kTile; r += 16) {
@@ -56,25 +76,45 @@ __global__ void __launch_bounds__(256) ingest_transpose_kernel(const uint8_t *__
     }
 }
 
-// The same with 16-byte global accesses (pointers and strides 16-byte
-// aligned) on 256 (time) x 64 (channel) tiles.  Thread (r, q) loads bytes
+// The same with 16-byte stores (output pointer and stride 16-byte aligned) on 256
+// (time) x 64 (channel) tiles.  Thread (r, q) loads bytes
 // [16q, 16q + 16) of time rows 4r .. 4r + 3 and transposes their 4 x 4 byte blocks in
 // registers (8 byte permutes per 16 bytes): 16 words of four samples, one per
 // channel, into the shared tile [channel][time].  Each half warp then reads 256
 // samples of a channel as 16-byte words and stores them, 256 contiguous bytes.
 // The tile's word column is XORed with 8 times the channel group, which keeps both
 // sides free of bank conflicts.  About 1.1 instructions per byte (four when each
-// byte was gathered from shared memory on its own).  4096 x 262144 samples: 458 ->
-// 346 us (6.2 TB/s of the 6.8 measured).  Edge tiles fall back to byte accesses.
+// byte was gathered from shared memory on its own).  Edge tiles fall back to byte accesses.
+// kVec: the input pointer and stride are 16-byte aligned too, and a thread's 16 bytes
+// are one load.  Otherwise they are five aligned words shifted into place, where those
+// words lie inside the matrix, or bytes.
 constexpr int kTileT16 = 256;
 
+// 16 bytes at src from aligned words; false where one would reach outside [lo, hi).
+__device__ __forceinline__ bool load16_shifted(const uint8_t *src, const uint8_t *lo,
+                                               const uint8_t *hi, uint32_t (&v)[4]) {
+    const unsigned sh = (unsigned)((uintptr_t)src & 3);
+    const uint8_t *a = src - sh;
+    if (a < lo || a + (sh ? 20 : 16) > hi) return false;
+    uint32_t w[5];
+#pragma unroll
+    for (int k = 0; k < 4; k++) w[k] = __ldg(reinterpret_cast<const uint32_t *>(a) + k);
+    w[4] = sh ? __ldg(reinterpret_cast<const uint32_t *>(a) + 4) : 0u;
+#pragma unroll
+    for (int k = 0; k < 4; k++) v[k] = __funnelshift_r(w[k], w[k + 1], 8 * sh);
+    return true;
+}
+
+template <bool kVec>
 __global__ void __launch_bounds__(256) ingest_transpose16_kernel(const uint8_t *__restrict__ in,
                                                                  int64_t in_stride, int64_t N,
                                                                  int C, uint8_t *__restrict__ out,
                                                                  int64_t out_stride) {
     __shared__ __align__(16) uint32_t tile[kTile][kTileT16 / 4];
-    const int64_t t0 = (int64_t)blockIdx.x * kTileT16;
-    const int c0 = blockIdx.y * kTile;
+    unsigned tt, ct;
+    tile_of(&tt, &ct);
+    const int64_t t0 = (int64_t)tt * kTileT16;
+    const int c0 = (int)ct * kTile;
     {
         const int q = threadIdx.x & 3, r = threadIdx.x >> 2;
         const int c = c0 + 16 * q;
@@ -83,21 +123,27 @@ __global__ void __launch_bounds__(256) ingest_transpose16_kernel(const uint8_t *
         for (int i = 0; i < 4; i++) {
             const int64_t t = t0 + 4 * r + i;
             const uint8_t *src = in + t * in_stride + c;
-            uint4 x = make_uint4(0u, 0u, 0u, 0u);
+            v[i][0] = v[i][1] = v[i][2] = v[i][3] = 0u;
             if (t < N) {
+                bool done = false;
                 if (c + 15 < C) {
-                    x = __ldcs(reinterpret_cast<const uint4 *>(src));
-                } else {
-                    uint32_t w[4] = {0u, 0u, 0u, 0u};
+                    if (kVec) {
+                        const uint4 x = __ldcs(reinterpret_cast<const uint4 *>(src));
+                        v[i][0] = x.x;
+                        v[i][1] = x.y;
+                        v[i][2] = x.z;
+                        v[i][3] = x.w;
+                        done = true;
+                    } else {
+                        done = load16_shifted(src, in, in + (N - 1) * in_stride + C, v[i]);
+                    }
+                }
+                if (!done) {
+#pragma unroll
                     for (int k = 0; k < 16; k++)
-                        if (c + k < C) w[k >> 2] |= (uint32_t)__ldg(src + k) << (8 * (k & 3));
-                    x = make_uint4(w[0], w[1], w[2], w[3]);
+                        if (c + k < C) v[i][k >> 2] |= (uint32_t)__ldg(src + k) << (8 * (k & 3));
                 }
             }
-            v[i][0] = x.x;
-            v[i][1] = x.y;
-            v[i][2] = x.z;
-            v[i][3] = x.w;
         }
 #pragma unroll
         for (int k = 0; k < 4; k++) {
@@ -144,13 +190,15 @@ extern "C" gsp_status gsp_ingest_transpose(const uint8_t *d_in, int64_t n_samp, 
     const bool words = ((((uintptr_t)d_in | (uintptr_t)d_out) & 3) == 0) && (in_stride % 4 == 0) &&
                        (out_stride % 4 == 0);
     dim3 grid((unsigned)tiles_t, (unsigned)tiles_c);
-    const bool v16 = ((((uintptr_t)d_in | (uintptr_t)d_out) & 15) == 0) && (in_stride % 16 == 0) &&
-                     (out_stride % 16 == 0);
-    if (v16) {
-        dim3 grid16((unsigned)((n_samp + kTileT16 - 1) / kTileT16), (unsigned)tiles_c);
-        ingest_transpose16_kernel<<<grid16, 256, 0, (cudaStream_t)stream>>>(
+    const bool out16 = ((uintptr_t)d_out & 15) == 0 && out_stride % 16 == 0;
+    const bool in16 = ((uintptr_t)d_in & 15) == 0 && in_stride % 16 == 0;
+    dim3 grid16((unsigned)((n_samp + kTileT16 - 1) / kTileT16), (unsigned)tiles_c);
+    if (out16 && in16)
+        ingest_transpose16_kernel<true><<<grid16, 256, 0, (cudaStream_t)stream>>>(
             d_in, in_stride, n_samp, nchan, d_out, out_stride);
-    }
+    else if (out16)
+        ingest_transpose16_kernel<false><<<grid16, 256, 0, (cudaStream_t)stream>>>(
+            d_in, in_stride, n_samp, nchan, d_out, out_stride);
     else
         ingest_transpose_kernel<<<grid, 256, 0, (cudaStream_t)stream>>>(d_in, in_stride, n_samp,
                                                                         nchan, d_out, out_stride,

@@ -158,3 +158,25 @@ def test_training_layers_consistent(gsp, n):
         assert (abs(g[at:at + cout] - db) <= (k + 8) * 2.0 ** -24 * abs(v).sum((0, 1, 2)) + 1e-30).all()
         at += cout
         act = t["a"].reshape(n, h, h, cout)
+
+
+@pytest.mark.parametrize("n,c,pad,off,out_off", [
+    (256, 320, 0, 0, 0),     # five channel tiles: a group of four and one alone
+    (257, 321, 2, 1, 0),     # input words shifted by 1, 2 and 3 bytes
+    (255, 80, 3, 2, 0),
+    (1, 16, 0, 3, 0),        # the only words would reach outside the matrix
+    (2, 17, 0, 0, 0),
+    (1030, 706, 0, 0, 0),
+    (513, 130, 4, 0, 0),
+    (300, 260, 16, 0, 1),    # output not aligned: the kernel of byte and word accesses
+])
+def test_ingest_alignments(gsp, n, c, pad, off, out_off):
+    rng = np.random.default_rng(n * c + off)
+    flat = torch.from_numpy(rng.integers(0, 256, n * (c + pad) + off, dtype=np.uint8)).cuda()
+    x = flat[off:].view(n, c + pad)
+    stride = (n + 15) // 16 * 16 + 16
+    buf = torch.full((c * stride + out_off,), 7, dtype=torch.uint8, device="cuda")
+    out = buf[out_off:].view(c, stride)
+    gsp.gsp_ingest_transpose(x, n, c, out)
+    assert torch.equal(out[:, :n], x[:, :c].t())
+    assert bool((out[:, n:] == 7).all()) and bool((buf[:out_off] == 7).all())
