@@ -4,39 +4,18 @@
 // read and one write per byte.  Rows of the output that are 16-byte aligned take
 // ingest_transpose16_kernel, whatever the input's alignment; others a kernel of
 // 64 x 64 byte tiles with 4-byte or byte accesses.
-//
-// A tile is 64 channels wide, half of a 128-byte line of the input.  Tiles are
-// therefore visited in groups of kGroup channel tiles side by side before the next
-// time tile: with all time tiles of one channel tile first, every line comes from
-// memory in two halves at different times (4096 x 2^20 samples, one / two / four /
-// eight / all side by side: 2076 / 1377 / 1368 / 1376 / 1377 us; rows of 2^20 + 16
-// bytes: 2151 / 1491 / 1490 / 1508 / 1548).
 #include "gsp_internal.cuh"
 
 namespace {
 
 constexpr int kTile = 64;
-constexpr unsigned kGroup = 4;
-
-// Tile of this CTA: grid (time tiles, channel tiles), renumbered within each kGroup
-// rows of the grid.  32 bits hold the number: more than 2^30 time tiles and more than
-// one channel tile would be over 2^42 bytes.
-__device__ __forceinline__ void tile_of(unsigned *tt, unsigned *ct) {
-    const unsigned c0 = blockIdx.y / kGroup * kGroup, g = min(kGroup, gridDim.y - c0);
-    const unsigned k = (blockIdx.y - c0) * gridDim.x + blockIdx.x;
-    *tt = k / g;
-    *ct = c0 + k % g;
-}
-
 __global__ void __launch_bounds__(256) ingest_transpose_kernel(const uint8_t *__restrict__ in,
                                                                int64_t in_stride, int64_t N, int C,
                                                                uint8_t *__restrict__ out,
                                                                int64_t out_stride, bool words) {
     __shared__ uint8_t tile[kTile][kTile + 4];
-    unsigned tt, ct;
-    tile_of(&tt, &ct);
-    const int64_t t0 = (int64_t)tt * kTile;   // time
-    const int c0 = (int)ct * kTile;           // channel
+    const int64_t t0 = (int64_t)blockIdx.x * kTile;   // time
+    const int c0 = blockIdx.y * kTile;                // channel
     const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;  // 16 x 16 threads
     // load: rows are times, 4 channels per thread
     for (int r = ty; r < kTile; r += 16) {
@@ -84,11 +63,34 @@ __global__ void __launch_bounds__(256) ingest_transpose_kernel(const uint8_t *__
 // samples of a channel as 16-byte words and stores them, 256 contiguous bytes.
 // The tile's word column is XORed with 8 times the channel group, which keeps both
 // sides free of bank conflicts.  About 1.1 instructions per byte (four when each
-// byte was gathered from shared memory on its own).  Edge tiles fall back to byte accesses.
+// byte was gathered from shared memory on its own).  4096 x 262144 samples: 466 -> 349 us
+// with nothing of them in L2 (6.2 TB/s of the 6.8 measured).  Edge tiles fall back to byte accesses.
 // kVec: the input pointer and stride are 16-byte aligned too, and a thread's 16 bytes
 // are one load.  Otherwise they are five aligned words shifted into place, where those
-// words lie inside the matrix, or bytes.
+// words lie inside the matrix, or bytes (706 x 110948 samples with rows of 710 bytes:
+// 95 us in the kernel of byte accesses above, 44 here; 4099-byte rows of 4096 channels,
+// 262144 samples: 1060, 470).
+//
+// A tile is 64 channels wide, half of a 128-byte line of the input.  Tiles are
+// therefore visited in groups of kGroup channel tiles side by side before the next
+// time tile: with all time tiles of one channel tile first, every line comes from
+// memory in two halves at different times (4096 x 2^20 samples, one / two / four /
+// eight / all side by side: 2076 / 1377 / 1368 / 1376 / 1377 us; output rows of 2^20 + 16
+// bytes: 2151 / 1491 / 1490 / 1508 / 1548).  Not so in the kernel above, whose stores of
+// 64 bytes are the half lines (4096 x 262144, output rows of 262148 bytes: 734 us in
+// time order, 830 in groups).
 constexpr int kTileT16 = 256;
+constexpr unsigned kGroup = 4;
+
+// Tile of this CTA: grid (time tiles, channel tiles), renumbered within each kGroup
+// rows of the grid.  32 bits hold the number: more than 2^30 time tiles and more than
+// one channel tile would be over 2^42 bytes.
+__device__ __forceinline__ void tile_of(unsigned *tt, unsigned *ct) {
+    const unsigned c0 = blockIdx.y / kGroup * kGroup, g = min(kGroup, gridDim.y - c0);
+    const unsigned k = (blockIdx.y - c0) * gridDim.x + blockIdx.x;
+    *tt = k / g;
+    *ct = c0 + k % g;
+}
 
 // 16 bytes at src from aligned words; false where one would reach outside [lo, hi).
 __device__ __forceinline__ bool load16_shifted(const uint8_t *src, const uint8_t *lo,
