@@ -258,6 +258,14 @@ __global__ void __launch_bounds__(kThreads, 1) dd_mma_kernel(const __grid_consta
             const int64_t t0 = tile * bt.T;
             const MmaFrame *fr = bt.frames + bt.foff[blk];
             const int nfr = bt.foff[blk + 1] - bt.foff[blk];
+            if (bt.add) {
+                // the series that the item adds to, towards L2: the epilogue waits for a
+                // round trip per 16 columns
+                const int d = blk * kKdm + dmi;
+                const int n = d < bt.ndm ? (int)min((int64_t)bt.T, bt.n_out - t0) : 0;
+                const int32_t *o = bt.out + (int64_t)min(d, bt.ndm - 1) * bt.out_stride + t0;
+                for (int j = 32 * tau; j < n; j += 256) asm volatile("prefetch.global.L2 [%0];" ::"l"(o + j));
+            }
             for (int f = 1; f < nfr; f++) {
                 // the frame's record, loaded ahead of its boundary
                 const int ne = (int)__ldg(&fr[f].e[dmi]), nrmax = __ldg(&fr[f].rmax);
@@ -788,7 +796,8 @@ bool mma_plan_tables(const int32_t *delays, int ndm, int C, bool rev, int npos, 
     return true;
 }
 
-int mma_split(const int32_t *delays, int ndm, int C, bool rev, int step, double other_rate) {
+int mma_split(const int32_t *delays, int ndm, int C, bool rev, int step, double other_rate,
+              double other_fixed) {
     const int nblk = (ndm + kKdm - 1) / kKdm;
     // the last block but one (complete, and as steep as any on a uniform grid)
     std::vector<int32_t> dl((size_t)C * kKdm);
@@ -797,7 +806,8 @@ int mma_split(const int32_t *delays, int ndm, int C, bool rev, int step, double 
     int32_t R[kKdm];
     int reach = 0;  // positions whose rows stay within a tile
     (void)block_frames(dl.data(), C, R, &frames, [&](int pos, int, int) { reach = pos + 1; });
-    double best = 0.9 * 16.0 * C / other_rate;  // clocks per sample of 16 trials: at least a tenth less
+    // clocks per sample of 16 trials: at least a twentieth less
+    double best = 0.95 * 16.0 * (C / other_rate + other_fixed);
     int npos = 0;
     size_t f = 0;
     double sum_r = 0.0;
@@ -815,7 +825,7 @@ int mma_split(const int32_t *delays, int ndm, int C, bool rev, int step, double 
         m.frames_per_block = (double)f;
         const int T = mma_tile_len(m.rmax);
         if (T < 512 || n < 256) continue;
-        const double c = mma_item_clocks(m, n, T) / T + 16.0 * rest / other_rate;
+        const double c = mma_item_clocks(m, n, T, true) / T + 16.0 * (rest / other_rate + other_fixed);
         if (c < best) {
             best = c;
             npos = n;
@@ -827,14 +837,20 @@ int mma_split(const int32_t *delays, int ndm, int C, bool rev, int step, double 
 int mma_tile_len(int rmax) { return std::max(0, (8 * kCols - rmax) & ~15); }
 
 // Measured on GB300: 165 clocks per channel at T + R = 1840 samples (the product alone
-// takes 115; the rest is the shared-memory port's, see above), 4300 per frame
-// boundary (drain, move, restart), 13,000 per item for the epilogue.
-double mma_item_clocks(const MmaShape &m, int nchan, int T) {
-    return nchan * (0.67 * ((T + m.mean_r) / 8.0 + 8.0) + 4.0) +
-           m.frames_per_block * (14.0 * T / 8.0 + 1300.0) + 14000.0;
+// takes 115; the rest is the shared-memory port's, see above) and not under 152 for a
+// shorter tile, 5,500 per frame boundary (drain, move, restart), 13,000 per item for the
+// epilogue, 8 per sample for reading the series that it adds to (17 without the lines
+// fetched ahead: 842 channels, 2062 trials 2046 us, 1956 with).  Within 4% of 25
+// launches of 325 to 3700 channels and 3 to 67 waves; the same without the floor and
+// with 4,000 per boundary was up to 40% low, and took grids of step 0.75 at 1000-1300
+// channels (2.50 ms) from the byte kernel (2.23).
+double mma_item_clocks(const MmaShape &m, int nchan, int T, bool add) {
+    return nchan * std::max(152.0, 0.67 * ((T + m.mean_r) / 8.0 + 8.0) + 4.0) +
+           m.frames_per_block * (14.0 * T / 8.0 + 2900.0) + 14000.0 + (add ? 8.0 * T : 0.0);
 }
 
-double mma_launch_clocks(const MmaShape &m, int nchan, int ndm, int64_t n_out, int num_sms, int *tile) {
+double mma_launch_clocks(const MmaShape &m, int nchan, int ndm, int64_t n_out, int num_sms, bool add,
+                         int *tile) {
     const int nblk = (ndm + kKdm - 1) / kKdm, tmax = mma_tile_len(m.rmax);
     *tile = 0;
     if (tmax < 16) return 1e30;
@@ -845,13 +861,13 @@ double mma_launch_clocks(const MmaShape &m, int nchan, int ndm, int64_t n_out, i
         const int T = std::min(tmax, (int)(((n_out + k - 1) / k + 15) & ~(int64_t)15));
         if (T < 256 && k > lo) break;
         const int64_t items = (n_out + T - 1) / T * nblk;
-        const double c = (double)((items + num_sms - 1) / num_sms) * mma_item_clocks(m, nchan, T);
+        const double c = (double)((items + num_sms - 1) / num_sms) * mma_item_clocks(m, nchan, T, add);
         if (*tile == 0 || c < best) {
             best = c;
             *tile = T;
         }
     }
-    return best;
+    return best + kLaunchClocks;
 }
 
 cudaError_t launch_dedisperse_mma(const BeamLaunch *beams, int nbeams, bool add, int num_sms, int *err,
@@ -897,7 +913,7 @@ cudaError_t launch_dedisperse_mma(const BeamLaunch *beams, int nbeams, bool add,
         const int64_t nt = (in.n_out + tmax - 1) / tmax;
         bt.T = std::min(tmax, (int)(((in.n_out + nt - 1) / nt + 15) & ~(int64_t)15));
         if (nbeams == 1)
-            (void)mma_launch_clocks(p->mma.shape, a.nchan, p->desc.ndm, in.n_out, num_sms, &bt.T);
+            (void)mma_launch_clocks(p->mma.shape, a.nchan, p->desc.ndm, in.n_out, num_sms, add, &bt.T);
         bt.ntiles = (in.n_out + bt.T - 1) / bt.T;
         bt.item0 = items;
         items += bt.ntiles * bt.nblk;

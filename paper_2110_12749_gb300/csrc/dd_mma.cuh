@@ -41,14 +41,19 @@ struct MmaShape {
 // npos of them.  false: a block's delays drift apart by more than a tile.
 bool mma_plan_tables(const int32_t *delays, int ndm, int C, bool rev, int npos, MmaTables *t);
 // How many positions to take where the rest (a multiple of step channels) is left to a
-// kernel of other_rate additions per clock and SM; 0 if that gains less than a tenth.
-int mma_split(const int32_t *delays, int ndm, int C, bool rev, int step, double other_rate);
+// kernel of other_rate additions per clock and SM and other_fixed clocks per sample of a
+// trial; 0 if that gains less than a twentieth.
+int mma_split(const int32_t *delays, int ndm, int C, bool rev, int step, double other_rate,
+              double other_fixed);
 // Longest tile (output samples) for a largest R.
 int mma_tile_len(int rmax);
 // Estimated SM clocks of one work item (16 DM trials x T samples x nchan channels).
-double mma_item_clocks(const MmaShape &m, int nchan, int T);
+// add: to a series that is there already.
+double mma_item_clocks(const MmaShape &m, int nchan, int T, bool add);
 
 // The same of a whole launch of one beam, and the tile length it is least at.
-double mma_launch_clocks(const MmaShape &m, int nchan, int ndm, int64_t n_out, int num_sms, int *tile);
+double mma_launch_clocks(const MmaShape &m, int nchan, int ndm, int64_t n_out, int num_sms, bool add,
+                         int *tile);
+constexpr double kLaunchClocks = 14000.0;  // of any launch, beside its work items
 
 }  // namespace gsp

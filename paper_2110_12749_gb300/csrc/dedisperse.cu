@@ -922,18 +922,23 @@ bool lists_ok(const TiledVariant &v, bool have_lists) { return !v.pre || have_li
 constexpr int kMmaMaxChannels = 65793;  // 255 nchan < 2^24: the FP32 sums are exact
 constexpr int kMmaMinTile = 256;        // shortest tile the tensor-core kernel is used at
 
-// Additions per clock and SM of the byte kernel's automatic variants (measured).
-double byte_rate(int variant) { return variant == kDefaultVariant ? 86.0 : (variant == 42 ? 78.0 : 60.0); }
+// Additions per clock and SM of the byte kernel's automatic variants, and the clocks of
+// a CTA's prologue and epilogue (measured: 289 to 3498 channels within 3%).
+double byte_rate(int variant) { return variant == kDefaultVariant ? 87.2 : (variant == 42 ? 81.0 : 60.0); }
+constexpr double kByteCtaClocks = 9000.0;
+// ... per sample of a trial.
+double byte_fixed(int variant) {
+    return kByteCtaClocks / (kVariants[variant].kdm * (128.0 * kVariants[variant].m - 4.0));
+}
 
-// Estimated SM clocks of a launch of one beam: waves of one CTA per SM, 13,000
-// clocks of prologue and epilogue per CTA (256 channels, 200 trials, 31,000 samples:
-// 186,000 measured, 188,000 estimated).
+// Estimated SM clocks of a launch of one beam, in waves of one CTA per SM.
 double byte_launch_clocks(int variant, int nchan, int ndm, int64_t n_out, int num_sms) {
     const TiledVariant &v = kVariants[variant];
     const int t_eff = 128 * v.m - 4;
     const int64_t items = (n_out + t_eff - 1) / t_eff * ((ndm + v.kdm - 1) / v.kdm);
     return (double)((items + num_sms - 1) / num_sms) *
-           ((double)nchan * v.kdm * t_eff / byte_rate(variant) + 13000.0);
+               ((double)nchan * v.kdm * t_eff / byte_rate(variant) + kByteCtaClocks) +
+           kLaunchClocks;
 }
 
 // The first variant of the automatic list that fits; -1 if none does.
@@ -1090,8 +1095,8 @@ bool plan_dedisperse_tiled(gsp_plan_s *p, TiledTables *tab) {
     if (tables(C)) {
         MmaShape &m = p->mma.shape;
         const int T = mma_tile_len(m.rmax);
-        const double byte_clk = 16.0 * T * C / byte_rate(variant);
-        const double mma_clk = T >= kMmaMinTile ? mma_item_clocks(m, C, T) : 1e30;
+        const double byte_clk = 16.0 * T * (C / byte_rate(variant) + byte_fixed(variant));
+        const double mma_clk = T >= kMmaMinTile ? mma_item_clocks(m, C, T, false) : 1e30;
         if (force_mma && T >= 16) {
             variant = kMmaVariant;
         } else if (mma_clk > 1.2 * byte_clk) {
@@ -1103,9 +1108,9 @@ bool plan_dedisperse_tiled(gsp_plan_s *p, TiledTables *tab) {
     }
     // A band of which only a part drifts slowly enough: the tensor-core kernel for that
     // part, the byte kernel for the whole stages of steep channels before it (2048
-    // channels, 500-3300 MHz, 3000 trials, 600011 samples: 26.7 -> 22.2 ms).
+    // channels, 500-3300 MHz, 3000 trials, 600011 samples: 26.7 -> 21.5 ms).
     if (!forced && !force_mma && variant != kMmaVariant) {
-        const int npos = mma_split(p->delays_h.data(), ndm, C, rev, 64, byte_rate(variant));
+        const int npos = mma_split(p->delays_h.data(), ndm, C, rev, 64, byte_rate(variant), byte_fixed(variant));
         if (npos > 0) {
             split = tables(npos) && mma_tile_len(p->mma.shape.rmax) >= kMmaMinTile;
             if (!split) tab->mma = MmaTables();
@@ -1275,7 +1280,7 @@ cudaError_t launch_dedisperse_batch(const BeamLaunch *beams, int nbeams, int var
         // one short beam: the byte kernel where its waves are estimated to end earlier
         const int bv = p->geom.byte_variant;
         if (nbeams > 1 || bv < 0 ||
-            mma_launch_clocks(p->mma.shape, C, ndm, n_out, num_sms, &T) <=
+            mma_launch_clocks(p->mma.shape, C, ndm, n_out, num_sms, false, &T) <=
                 byte_launch_clocks(bv, C, ndm, n_out, num_sms))
             return launch_dedisperse_mma(beams, nbeams, false, num_sms, err, s, nlaunch);
         variant = bv;
@@ -1283,7 +1288,7 @@ cudaError_t launch_dedisperse_batch(const BeamLaunch *beams, int nbeams, int var
                (!beams[0].bsum || p->desc.block_len >= kMmaMinBlock)) {
         // the steep channels' sums first, then the others' added to them
         const int n1 = p->mma.shape.npos;
-        if (mma_launch_clocks(p->mma.shape, n1, ndm, n_out, num_sms, &T) +
+        if (mma_launch_clocks(p->mma.shape, n1, ndm, n_out, num_sms, true, &T) +
                 byte_launch_clocks(variant, C - n1, ndm, n_out, num_sms) <
             byte_launch_clocks(variant, C, ndm, n_out, num_sms)) {
             BeamLaunch steep = beams[0];
