@@ -766,7 +766,7 @@ bool mma_plan_tables(const int32_t *delays, int ndm, int C, bool rev, int npos, 
     std::vector<std::vector<MmaFrame>> fr((size_t)nblk);
     std::vector<double> sum_r((size_t)nblk, 0.0);
     std::atomic<bool> fits{true};
-    const bool ran = parallel_ranges(nblk, std::max(1, 100000 / (npos * kKdm)), [&](int64_t b0, int64_t b1) {
+    const bool ran = parallel_ranges(nblk, std::max(1, 30000 / (npos * kKdm)), [&](int64_t b0, int64_t b1) {
         std::vector<int32_t> dl((size_t)npos * kKdm);
         for (int64_t b = b0; b < b1 && fits; b++) {
             block_delays(delays, ndm, C, rev, npos, (int)b, dl.data());

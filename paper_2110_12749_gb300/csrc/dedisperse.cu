@@ -131,7 +131,8 @@ struct TiledArgs {
     int *err;      // set to 1 if a bounded wait gave up
     int64_t items;
     long long budget;  // SM clock cycles a pipeline wait may take before it gives up
-    int st0, st1;      // stages of channels to sum (all of them, or the steep ones)
+    int pitch, fpitch;  // rows of the delay tables and of fcnt (longer than nchan where only a
+                        // band's steep channels are summed: the tables start at the first)
     int starve;        // failure-path test: the producer issues nothing, so every stage wait
                        // runs out (no copy is ever in flight)
 };
@@ -372,8 +373,8 @@ __global__ void __launch_bounds__((KDM / KW + 1) * 32, (KDM / KW + 1) * 32 <= 25
         decode_item(a, item, &bi, &tile, &blk);
         const BeamTile &bt = a.beam[bi];
         const int64_t t0 = tile * kTEff;
-        const int32_t *bmin = bt.blkmin + (int64_t)blk * a.nchan;
-        for (int st = a.st0; st < a.st1 && ok; st++, gst++) {
+        const int32_t *bmin = bt.blkmin + (int64_t)blk * a.pitch;
+        for (int st = 0; st < nst && ok; st++, gst++) {
             if (wrapped) {
                 const bool w = ptx::mbar_wait(empty(slot), rpar ^ 1u, a.budget);
                 if (!__all_sync(0xffffffffu, w)) {
@@ -459,7 +460,7 @@ __global__ void __launch_bounds__((KDM / KW + 1) * 32, (KDM / KW + 1) * 32 <= 25
     const BeamTile &bt = a.beam[bi];
     const int64_t t0 = tile * kTEff;
     const int dm0 = blk * KDM;
-    const int32_t *bmin = bt.blkmin + (int64_t)blk * a.nchan;
+    const int32_t *bmin = bt.blkmin + (int64_t)blk * a.pitch;
     const int dmw = dm0 + warp * kKW;
     uint32_t acc[kKW][kM][4];
     uint32_t E[kKW][4][kM], O[kKW][4][kM];
@@ -480,25 +481,25 @@ __global__ void __launch_bounds__((KDM / KW + 1) * 32, (KDM / KW + 1) * 32 <= 25
     // delays of the next stage are loaded one stage ahead (hides L2 latency)
     // PRE: nx_dl holds the packed (delay << 8) | list position instead of the delay
     const int32_t *dtab = PRE ? bt.dpos : bt.delays;
-    const uint32_t *fcrow = PRE ? bt.fcnt + (int64_t)min(dmw, bt.ndm - 1) * nst : nullptr;
+    const uint32_t *fcrow = PRE ? bt.fcnt + (int64_t)min(dmw, bt.ndm - 1) * a.fpitch : nullptr;
     int nx_min[kH], nx_dl[kKW][kH];
-    uint32_t nx_fc = PRE ? fcrow[a.st0] : 0u;
+    uint32_t nx_fc = PRE ? fcrow[0] : 0u;
 #pragma unroll
     for (int h = 0; h < kH; h++) {
-        const int c0 = a.st0 * kCB + h * 32 + lane;
+        const int c0 = h * 32 + lane;
         const bool v0 = c0 < a.nchan;
         nx_min[h] = v0 ? bmin[c0] : 0;
 #pragma unroll
         for (int i = 0; i < kKW; i++)
-            nx_dl[i][h] = v0 ? dtab[(int64_t)min(dmw + i, bt.ndm - 1) * a.nchan + c0] : 0;
+            nx_dl[i][h] = v0 ? dtab[(int64_t)min(dmw + i, bt.ndm - 1) * a.pitch + c0] : 0;
     }
 
-    for (int st = a.st0; st < a.st1; st++) {
+    for (int st = 0; st < nst; st++) {
         int cur_min[kH], cur_dl[kKW][kH];
         // the same word in every lane; a warp reduction makes that visible to the compiler,
         // so the family loops below branch on a warp-uniform count
         const uint32_t cur_fc = PRE ? __reduce_or_sync(0xffffffffu, nx_fc) : 0u;
-        if (PRE && st + 1 < a.st1) nx_fc = fcrow[st + 1];
+        if (PRE && st + 1 < nst) nx_fc = fcrow[st + 1];
 #pragma unroll
         for (int h = 0; h < kH; h++) {
             cur_min[h] = nx_min[h];
@@ -509,7 +510,7 @@ __global__ void __launch_bounds__((KDM / KW + 1) * 32, (KDM / KW + 1) * 32 <= 25
             nx_min[h] = vn ? bmin[cn] : 0;
 #pragma unroll
             for (int i = 0; i < kKW; i++)
-                nx_dl[i][h] = vn ? dtab[(int64_t)min(dmw + i, bt.ndm - 1) * a.nchan + cn] : 0;
+                nx_dl[i][h] = vn ? dtab[(int64_t)min(dmw + i, bt.ndm - 1) * a.pitch + cn] : 0;
         }
         int cnt[kKW][4];
 #pragma unroll
@@ -678,10 +679,10 @@ __global__ void __launch_bounds__((KDM / KW + 1) * 32, (KDM / KW + 1) * 32 <= 25
             rpar ^= 1u;
         }
 
-        if (MF && ((st + 1) % kFlushStages == 0 || st == a.st1 - 1)) {
+        if (MF && ((st + 1) % kFlushStages == 0 || st == nst - 1)) {
 #pragma unroll
             for (int i = 0; i < kKW; i++) flush_merged<kM>(E[i], O[i], acc[i], lane);
-        } else if (FF && st == a.st1 - 1) {
+        } else if (FF && st == nst - 1) {
 #pragma unroll
             for (int i = 0; i < kKW; i++) {
                 flush_family<0, kM, ACC>(E[i][0], O[i][0], acc[i], lane);
@@ -689,7 +690,7 @@ __global__ void __launch_bounds__((KDM / KW + 1) * 32, (KDM / KW + 1) * 32 <= 25
                 flush_family<2, kM, ACC>(E[i][2], O[i][2], acc[i], lane);
                 flush_family<3, kM, ACC>(E[i][3], O[i][3], acc[i], lane);
             }
-        } else if (!MF && !FF && ((st + 1) % kFlushStages == 0 || st == a.st1 - 1)) {
+        } else if (!MF && !FF && ((st + 1) % kFlushStages == 0 || st == nst - 1)) {
 #pragma unroll
             for (int i = 0; i < kKW; i++) {
                 uint32_t sp[kM][3];
@@ -968,7 +969,7 @@ void plan_phase_lists(const gsp_plan_s *p, int cb, std::vector<int32_t> *dpos,
     if (p->max_delay >= ((int64_t)1 << 23)) return;  // packed delay field is 23 bits
     dpos->resize((size_t)ndm * C);
     fcnt->resize((size_t)ndm * nst);
-    const bool ran = parallel_ranges(ndm, std::max(1, 200000 / C), [&](int64_t d0, int64_t d1) {
+    const bool ran = parallel_ranges(ndm, std::max(1, 50000 / C), [&](int64_t d0, int64_t d1) {
         for (int64_t d = d0; d < d1; d++) {
             const int32_t *dl = p->delays_h.data() + (size_t)d * C;
             int32_t *pos = dpos->data() + (size_t)d * C;
@@ -1225,15 +1226,15 @@ cudaError_t launch_bytes(const BeamLaunch *beams, int nbeams, int variant, bool 
         const BeamLaunch &in = beams[b];
         const gsp_plan_s *p = in.plan;
         BeamTile &bt = a.beam[b];
-        bt.x = in.x;
+        bt.x = in.x + (int64_t)c0 * in.x_stride;
         bt.x_stride = in.x_stride;
         bt.n_in = in.n_in;
         bt.n_out = in.n_out;
-        bt.delays = p->d_delays;
-        bt.blkmin = p->d_blkmin[o];
-        bt.dpos = p->d_dpos[ci];
-        bt.fcnt = p->d_fcnt[ci];
-        bt.stspread = p->d_stspread[o][ci];
+        bt.delays = p->d_delays + c0;
+        bt.blkmin = p->d_blkmin[o] + c0;
+        bt.dpos = v.pre ? p->d_dpos[ci] + c0 : nullptr;
+        bt.fcnt = v.pre ? p->d_fcnt[ci] + c0 / v.cb : nullptr;
+        bt.stspread = p->d_stspread[o][ci] + c0 / v.cb;
         bt.out = in.out;
         bt.out_stride = in.out_stride;
         bt.bsum = in.bsum;
@@ -1249,14 +1250,14 @@ cudaError_t launch_bytes(const BeamLaunch *beams, int nbeams, int variant, bool 
         items += bt.ntiles * bt.nblk;
     }
     a.nbeams = nbeams;
-    a.nchan = nchan;
+    a.nchan = c1 - c0;
+    a.pitch = nchan;
+    a.fpitch = (nchan + v.cb - 1) / v.cb;
     a.win = f.win;
     a.stages = f.stages;
     a.one = 1u;
     a.err = err;
     a.items = items;
-    a.st0 = c0 / v.cb;
-    a.st1 = (c1 + v.cb - 1) / v.cb;
     a.budget = beams[0].plan->wait_budget;
     a.starve = beams[0].plan->wait_starve;
     int64_t grid = persistent ? std::min<int64_t>(items, (int64_t)num_sms * f.ctas_per_sm) : items;

@@ -59,7 +59,7 @@ gsp_status compute_delays(const gsp_plan_desc *d, const std::vector<double> &dms
     }
     std::vector<double> margins(dms.size(), 1.0);
     std::atomic<bool> valid{true};
-    const bool ran = gsp::parallel_ranges((int64_t)dms.size(), std::max<int64_t>(1, 200000 / C), [&](int64_t i0, int64_t i1) {
+    const bool ran = gsp::parallel_ranges((int64_t)dms.size(), std::max<int64_t>(1, 50000 / C), [&](int64_t i0, int64_t i1) {
         for (int64_t i = i0; i < i1; i++) {
             const double dm = dms[i];
             double least = 1.0;
