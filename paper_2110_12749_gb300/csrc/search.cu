@@ -557,7 +557,9 @@ __global__ void __launch_bounds__(256, 3) boxcar_block_kernel(
     constexpr int B = kChunk, NW = kNumDefaultWidths;
     static_assert(B == 4 * kBoxThreads, "four samples per thread");
     __shared__ __align__(16) uint32_t sP[2][B + kTail];  // exclusive prefix sums of a block and the next
-    __shared__ uint32_t wtot[kBoxThreads / 32];
+    // warps' totals, by the parity of the block: the first two scans follow each other with
+    // no barrier between a warp's reads of the one and another's writes of the next
+    __shared__ uint32_t wtot[2][kBoxThreads / 32];
     __shared__ Peak wbest[kBoxThreads / 32];
     __shared__ float s_scale[NW];
     __shared__ int s_width[NW];
@@ -609,7 +611,10 @@ __global__ void __launch_bounds__(256, 3) boxcar_block_kernel(
         return u < last || (u < nb && 4 * tid < kTail) ? __ldg(d4 + (int64_t)u * (B / 4))
                                                        : make_int4(0, 0, 0, 0);
     };
-    // prefix sums of block u (loaded as v) into its buffer and behind block u - 1's
+    // prefix sums of block u (loaded as v) into its buffer and behind block u - 1's.  The
+    // barrier in here separates this scan's writes of wtot from its reads, and the reads
+    // of scan(u - 1) from the writes of scan(u + 1), which use the same half; it also ends the
+    // search of block u - 2, whose buffer is rewritten, and its reads of wbest.
     auto scan = [&](int u, const int4 &v, const BlockParam &q) {
         const uint32_t m = q.good ? ~0u : 0u;
         const uint32_t y0 = (uint32_t)(v.x - q.m) & m, y1 = (uint32_t)(v.y - q.m) & m;
@@ -621,12 +626,12 @@ __global__ void __launch_bounds__(256, 3) boxcar_block_kernel(
             const uint32_t a = __shfl_up_sync(0xffffffffu, incl, o);
             if (lane >= o) incl += a;
         }
-        if (lane == 31) wtot[wid] = incl;
+        if (lane == 31) wtot[u & 1][wid] = incl;
         __syncthreads();
         uint32_t pre = carry + incl - tot, all = 0;
 #pragma unroll
         for (int w = 0; w < kBoxThreads / 32; w++) {
-            const uint32_t a = wtot[w];
+            const uint32_t a = wtot[u & 1][w];
             pre += w < wid ? a : 0u;
             all += a;
         }

