@@ -60,6 +60,7 @@ constexpr int kAWarp = 4;              // 4: write A (warps 0-3 move the rows of
 constexpr int kWideWarp = 8;           // 11: widen the channels in turn (16.1 ms on a
                                        // 131072-sample chunk; 8: 16.6, 10: 16.5, 12: 17.0)
 constexpr int kWideWarps = 11;
+static_assert(kWideWarps <= 2 * kChunk, "a widening warp leaves out one chunk at most");
 constexpr int kMmaWarp = kWideWarp + kWideWarps;  // issue the products (one lane)
 constexpr int kCopyWarp = kMmaWarp + 1;           // 2: copy the channels' windows of the chunks in turn
 constexpr int kCopyWarps = 2;
@@ -475,8 +476,13 @@ __global__ void __launch_bounds__(kThreads, 1) dd_mma_kernel(const __grid_consta
                     nbase = np < C ? __ldg(base + np) : 0;
                     nrm = __ldg(crmax + np / kChunk);
                 }
-                const bool landed = ptx::mbar_wait(raw_full(slot), par, a.budget) &&
-                                    ptx::mbar_wait(slot_empty(slot), par ^ 1u, a.budget);
+                // in this order: a warp that had no channel of this slot's last chunk may come
+                // here before that chunk's copy has landed, and the parity of raw_full would
+                // then read as complete a round early.  The slot's products of that chunk are
+                // done only after its copy has been read, so raw_full has moved on by then.  (A
+                // warp leaves out one chunk at most, so slot_empty is never two rounds behind.)
+                const bool landed = ptx::mbar_wait(slot_empty(slot), par ^ 1u, a.budget) &&
+                                    ptx::mbar_wait(raw_full(slot), par, a.budget);
                 if (!__all_sync(0xffffffffu, landed)) {
                     ok = false;
                     break;

@@ -40,3 +40,28 @@ def test_block_aligned_search_repeats(gsp, rows, nblk):
         gsp.gsp_search_series(plan, D, n)
         got, m, _ = gsp.gsp_candidates(plan)
         assert m == total and (got == want).all()
+
+
+@pytest.mark.parametrize("nchan,ndm,n_in", [(512, 32, 1 << 20), (24, 40, 1 << 21), (100, 16, 1 << 21), (9, 33, 1 << 20)])
+def test_tensor_core_dedispersion_repeats(gsp, monkeypatch, nchan, ndm, n_in):
+    """Rings of a few chunks per item, inputs cold in L2 and far apart: every pass of the
+    tensor-core kernel equals the byte kernel."""
+    g = torch.Generator(device="cuda")
+    g.manual_seed(nchan)
+    x = torch.randint(0, 256, (nchan, n_in), dtype=torch.uint8, device="cuda", generator=g)
+    cold = torch.empty(1 << 28, dtype=torch.uint8, device="cuda")
+    want = None
+    for variant in (32, gsp.gsp_dedisperse_variants()[0] - 1):
+        monkeypatch.setenv("GSP_DD_VARIANT", str(variant))
+        d, keep = gsp.make_desc(nchan, 1200.0, 1500.0, 1e-4, n_in, ndm=ndm, dm_step=0.7, block_len=4096)
+        plan = gsp.gsp_plan_create(d, keep)
+        assert gsp.gsp_dedisperse_variants(plan)[1] == variant
+        n_out = gsp.gsp_plan_nout(plan, n_in)
+        out = torch.zeros((ndm, (n_out + 3) // 4 * 4), dtype=torch.int32, device="cuda")
+        for _ in range(1 if want is None else 25):
+            out.zero_()
+            cold.fill_(1)
+            gsp.gsp_dedisperse(plan, x, n_in, out)
+            if want is None:
+                want = out.clone()
+            assert torch.equal(out, want)
