@@ -605,19 +605,16 @@ __global__ void __launch_bounds__(kThreads, 1) dd_mma_kernel(const __grid_consta
             mma_decode(a, item, &bi, &tile, &blk);
             const MmaBeam &bt = a.beam[bi];
             const int T = bt.T;
-            // positions relative to the tile's start; the input is [in0, in1), and whole
-            // 16-byte pieces of it end at in16
+            // sample positions of the row, in 64 bits: a delay may be up to 2^31 - 1.  t0 is a
+            // multiple of 16; whole 16-byte pieces of the input end at in16
             const int64_t t0 = tile * T;
-            const int in0 = (int)max(-t0, (int64_t)-(1 << 30));
-            const int in1 = (int)min(bt.n_in - t0, (int64_t)1 << 30);
-            const int in16 = (int)min((bt.n_in & ~(int64_t)15) - t0, (int64_t)1 << 30);
-            const int tl = (int)(t0 & 15);
+            const int64_t in16 = bt.n_in & ~(int64_t)15;
             const int32_t *base = bt.base + (int64_t)blk * C;
             const int32_t *crmax = bt.crmax + (int64_t)blk * nchunk;
             const int k = lane;  // channel of the chunk (lanes 0..7)
             int ch = (grp + kCopyWarps - (int)(g % kCopyWarps)) % kCopyWarps;
             const int64_t step = (bt.rev ? -1 : 1) * bt.x_stride;
-            const uint8_t *row = bt.x + t0 + (bt.rev ? (int64_t)(C - 1) * bt.x_stride : 0) +
+            const uint8_t *row = bt.x + (bt.rev ? (int64_t)(C - 1) * bt.x_stride : 0) +
                                  step * (ch * kChunk + k);
             int nbase = k < kChunk && ch * kChunk + k < C ? __ldg(base + ch * kChunk + k) : 0;
             int nrm = ch < nchunk ? __ldg(crmax + ch) : 0;
@@ -626,7 +623,7 @@ __global__ void __launch_bounds__(kThreads, 1) dd_mma_kernel(const __grid_consta
                 const int slot = (int)(gc % kSlots);
                 const int pos = ch * kChunk + k;
                 const bool in = k < kChunk && pos < C;
-                const int s = nbase;                         // first sample
+                const int64_t s = t0 + nbase;                   // first sample
                 const int need = 8 * (frame_cols(T, nrm) + 1);  // samples from it
                 if (ch + kCopyWarps < nchunk) {
                     const int np = pos + kCopyWarps * kChunk;
@@ -635,10 +632,11 @@ __global__ void __launch_bounds__(kThreads, 1) dd_mma_kernel(const __grid_consta
                 }
                 // bytes [lo, hi) of the channel's row; the samples before the input (only
                 // columns of t < 0 take them) and past its end are left as they are
-                const int off = (s + tl) & 15, w0 = s - off;  // the window starts 16-byte aligned
-                const int lo = max(w0, in0);
-                const int hi = min(w0 + ((off + need + 15) & ~15), in1);
-                const int hi16 = min(hi, in16);
+                const int off = (int)(s & 15);
+                const int64_t w0 = s - off;  // the window starts 16-byte aligned
+                const int64_t lo = max(w0, (int64_t)0);
+                const int64_t hi = min(w0 + ((off + need + 15) & ~15), bt.n_in);
+                const int64_t hi16 = min(hi, in16);
                 const uint32_t bytes = in && hi16 > lo ? (uint32_t)(hi16 - lo) & ~15u : 0u;
                 const uint32_t tot = __reduce_add_sync(0xffffffffu, bytes);
                 if (!__all_sync(0xffffffffu, ptx::mbar_wait(raw_empty(slot), ((gc / kSlots) & 1u) ^ 1u,
@@ -648,7 +646,7 @@ __global__ void __launch_bounds__(kThreads, 1) dd_mma_kernel(const __grid_consta
                 }
                 const uint32_t dst = (uint32_t)(slot * kRawSlot + k * kRawPitch);
                 if (in && hi > hi16)  // the last bytes of the input
-                    for (int i = max(lo, hi16); i < hi; i++) raw[dst + (uint32_t)(i - w0)] = row[i];
+                    for (int64_t i = max(lo, hi16); i < hi; i++) raw[dst + (uint32_t)(i - w0)] = row[i];
                 __syncwarp();
                 if (lane == 0) ptx::mbar_arrive_expect_tx(raw_full(slot), tot);
                 __syncwarp();

@@ -65,3 +65,26 @@ def test_tensor_core_dedispersion_repeats(gsp, monkeypatch, nchan, ndm, n_in):
             if want is None:
                 want = out.clone()
             assert torch.equal(out, want)
+
+
+@pytest.mark.parametrize("first", [(1 << 30) - 600, (1 << 30) + 12345, (1 << 31) - 100])
+def test_delays_beyond_30_bits(gsp, monkeypatch, first):
+    """Delays around 2^30 samples and up to the largest one accepted, trials close together
+    (so that the tensor-core kernel takes them): the sums of two channels, exactly."""
+    monkeypatch.setenv("GSP_DD_VARIANT", str(gsp.gsp_dedisperse_variants()[0] - 1))
+    ndm, n_out = 17, 5000
+    delays = np.zeros((ndm, 2), np.int32)
+    delays[:, 0] = first + 5 * np.arange(ndm)
+    n_in = int(delays.max()) + n_out
+    g = torch.Generator(device="cuda")
+    g.manual_seed(1)
+    x = torch.randint(0, 256, (2, (n_in + 15) // 16 * 16), dtype=torch.uint8, device="cuda", generator=g)
+    d, keep = gsp.make_desc(2, 1200.0, 1500.0, 1e-4, n_in, delays=delays, block_len=1 << 16,
+                            window_len=1 << 20, max_cands=16)
+    plan = gsp.gsp_plan_create(d, keep)
+    assert gsp.gsp_dedisperse_variants(plan)[1] == gsp.gsp_dedisperse_variants()[0] - 1
+    out = torch.full((ndm, n_out), -7, dtype=torch.int32, device="cuda")
+    gsp.gsp_dedisperse(plan, x, n_in, out)
+    for i in range(ndm):
+        a = int(delays[i, 0])
+        assert torch.equal(out[i], x[0, a:a + n_out].int() + x[1, :n_out].int()), i
