@@ -88,3 +88,41 @@ def test_delays_beyond_30_bits(gsp, monkeypatch, first):
     for i in range(ndm):
         a = int(delays[i, 0])
         assert torch.equal(out[i], x[0, a:a + n_out].int() + x[1, :n_out].int()), i
+
+
+@pytest.mark.parametrize("nchan,values", [
+    (65793, (255, 255)),     # the most channels the kernel takes: 2^24 - 1 in every sample
+    (65792, (251, 255)),
+    (50001, (128, 255)),     # sums above 2^23 whose low bits vary
+    (33000, (254, 255)),
+    (65793, (0, 1)),
+])
+@pytest.mark.parametrize("descending", [False, True])
+def test_tensor_core_sums_to_24_bits(gsp, monkeypatch, nchan, values, descending):
+    """The FP32 accumulators hold whole numbers below 2^24: sums up to the limit are exact,
+    and so are the block sums taken from them."""
+    mma = gsp.gsp_dedisperse_variants()[0] - 1
+    monkeypatch.setenv("GSP_DD_VARIANT", str(mma))
+    ndm, n_out = 17, 2100
+    pos = np.arange(nchan) if descending else np.arange(nchan)[::-1]
+    delays = (pos[None, :] * (3 + np.arange(ndm)[:, None]) // 16384).astype(np.int32)
+    n_in = n_out + int(delays.max())
+    g = torch.Generator(device="cuda")
+    g.manual_seed(nchan)
+    x = torch.randint(values[0], values[1] + 1, (nchan, (n_in + 15) // 16 * 16), dtype=torch.uint8,
+                      device="cuda", generator=g)
+    d, keep = gsp.make_desc(nchan, 1200.0, 1500.0, 1e-4, n_in, delays=delays, freq_descending=descending)
+    plan = gsp.gsp_plan_create(d, keep)
+    assert gsp.gsp_dedisperse_variants(plan)[1] == mma
+    out = torch.full((ndm, n_out), -7, dtype=torch.int32, device="cuda")
+    gsp.gsp_search(plan, x, n_in, 0, out)
+    fused = gsp.gsp_search_stats(plan, n_out)
+    for i in range(ndm):
+        ref = torch.zeros(n_out, dtype=torch.int64, device="cuda")
+        for v in np.unique(delays[i]):
+            c = np.nonzero(delays[i] == v)[0]
+            ref += x[c[0]:c[-1] + 1, int(v):int(v) + n_out].sum(0, dtype=torch.int64)
+        assert torch.equal(out[i].long(), ref), i
+    gsp.gsp_search_series(plan, out, n_out)
+    plain = gsp.gsp_search_stats(plan, n_out)
+    assert (fused["sigma_b"] == plain["sigma_b"]).all() and (fused["bad"] == plain["bad"]).all()
