@@ -66,7 +66,7 @@ gsp_status enqueue(gsp_batch_s *b, const gsp_beam_input *in, int variant, cudaSt
         int64_t stride = 0;
         unsigned long long *bsum = nullptr;
         gsp_status st = gsp::plan_check_input(p, in[i].d_x, in[i].n_in, in[i].x_stride, &n_out[i]);
-        if (st == GSP_OK) st = gsp::plan_prepare_search(p, n_out[i], &D, &stride, &bsum);
+        if (st == GSP_OK) st = gsp::plan_prepare_search(p, n_out[i], variant, &D, &stride, &bsum);
         if (st != GSP_OK) return st;
         if (bsum && cudaMemsetAsync(bsum, 0, (size_t)p->desc.ndm * p->nb_max * 3 * sizeof(*bsum), s) !=
                         cudaSuccess)
@@ -121,7 +121,7 @@ float time_variant(gsp_batch_s *b, const gsp_beam_input *in, int v, cudaStream_t
         int32_t *D = nullptr;
         unsigned long long *bsum = nullptr;
         if (gsp::plan_check_input(p, in[i].d_x, in[i].n_in, in[i].x_stride, &n_out) != GSP_OK ||
-            gsp::plan_prepare_search(p, n_out, &D, &stride, &bsum) != GSP_OK)
+            gsp::plan_prepare_search(p, n_out, v, &D, &stride, &bsum) != GSP_OK)
             return -1.f;
         const int64_t n = std::min<int64_t>(n_out, kTuneSamples);
         bl[i] = gsp::BeamLaunch{p, in[i].d_x, n + p->max_delay, in[i].x_stride, n, D, stride,

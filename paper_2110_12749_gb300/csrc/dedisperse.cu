@@ -1125,6 +1125,10 @@ bool plan_dedisperse_tiled(gsp_plan_s *p, TiledTables *tab) {
 
 int dedisperse_num_variants() { return kNumVariants + 1; }
 
+int dedisperse_min_block(int variant) {
+    return variant == kMmaVariant ? kMmaMinBlock : 128 * kVariants[variant].m - 4;
+}
+
 int dedisperse_tune_candidates(const int **list) {
     *list = kTuneList;
     return (int)(sizeof(kTuneList) / sizeof(kTuneList[0]));
@@ -1151,7 +1155,6 @@ void dedisperse_set_variant(gsp_plan_s *p, int variant) {
         DDGeom &g = p->geom;
         g.kdm = 16;
         g.t_cta = mma_tile_len(p->mma.shape.rmax);
-        g.t_eff = kMmaMinBlock;  // search blocks at least this long have their sums fused
         g.cb = 8;
         g.win = g.stages = g.smem = 0;
         g.ctas_per_sm = 1;
@@ -1165,7 +1168,6 @@ void dedisperse_set_variant(gsp_plan_s *p, int variant) {
     DDGeom &g = p->geom;
     g.kdm = v.kdm;
     g.t_cta = 128 * v.m;
-    g.t_eff = 128 * v.m - 4;
     g.cb = v.cb;
     g.win = f.win;
     g.stages = f.stages;

@@ -199,10 +199,12 @@ gsp_status ensure_scratch_D(gsp_plan_s *p, int64_t n_out) {
     return GSP_OK;
 }
 
-// Block sums are fused into the tiled kernel when it can produce them (a
-// tile of 508 samples then touches at most two search blocks).
-bool fused_stats(const gsp_plan_s *p) {
-    return !p->simple_dd && p->d_bsum != nullptr && p->desc.block_len >= p->geom.t_eff;
+// Block sums are fused into the dedispersion kernel when the variant that is launched
+// can produce them: search blocks at least as long as a byte variant's tile (which then
+// touches at most two of them), or as the tensor-core kernel's smallest block.
+bool fused_stats(const gsp_plan_s *p, int variant) {
+    return !p->simple_dd && p->d_bsum != nullptr &&
+           p->desc.block_len >= gsp::dedisperse_min_block(variant);
 }
 
 gsp_status run_dedisperse(gsp_plan_s *p, const uint8_t *x, int64_t n_in, int64_t x_stride,
@@ -266,14 +268,14 @@ cudaError_t ensure_kernel_smem(const void *fn, int smem, bool max_carveout) {
 }
 
 // Used by the batch module: make sure the plan's series scratch exists and
-// tell whether block sums can be fused into the tiled dedispersion kernel.
-gsp_status plan_prepare_search(gsp_plan_s *p, int64_t n_out, int32_t **D, int64_t *stride,
-                               unsigned long long **bsum) {
+// tell whether block sums can be fused into dedispersion variant `variant`.
+gsp_status plan_prepare_search(gsp_plan_s *p, int64_t n_out, int variant, int32_t **D,
+                               int64_t *stride, unsigned long long **bsum) {
     gsp_status st = ensure_scratch_D(p, n_out);
     if (st != GSP_OK) return st;
     *D = p->d_D;
     *stride = (n_out + 3) & ~(int64_t)3;
-    *bsum = (fused_stats(p) && n_out / p->desc.block_len > 0) ? p->d_bsum : nullptr;
+    *bsum = (fused_stats(p, variant) && n_out / p->desc.block_len > 0) ? p->d_bsum : nullptr;
     return GSP_OK;
 }
 
@@ -514,7 +516,7 @@ gsp_status gsp_search(gsp_plan_t p, const uint8_t *d_x, int64_t n_in, int64_t x_
     p->launches = 0;
     unsigned long long *bsum = nullptr;
     const int64_t nb = n_out / p->desc.block_len;
-    if (fused_stats(p) && nb > 0) {
+    if (fused_stats(p, p->geom.variant) && nb > 0) {
         bsum = p->d_bsum;
         GSP_CK(cudaMemsetAsync(bsum, 0, (size_t)p->desc.ndm * p->nb_max * 3 * sizeof(*bsum), s));
     }
@@ -707,7 +709,7 @@ gsp_status gsp_search_host(gsp_plan_t p, const uint8_t *h_x, int64_t n_in, int64
     const int64_t stride = (n_out + 3) & ~(int64_t)3;
     p->launches = 0;
     unsigned long long *bsum = nullptr;
-    if (fused_stats(p) && n_out / B > 0) {
+    if (fused_stats(p, p->geom.variant) && n_out / B > 0) {
         bsum = p->d_bsum;
         GSP_CK(cudaMemsetAsync(bsum, 0, (size_t)p->desc.ndm * p->nb_max * 3 * sizeof(*bsum), s));
     }

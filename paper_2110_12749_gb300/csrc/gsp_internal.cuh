@@ -77,8 +77,7 @@ inline int cb_index(int cb) { return cb == 32 ? 1 : 0; }
 // Tile geometry of the performance dedispersion kernel, chosen per plan.
 struct DDGeom {
     int kdm = 0;       // DM trials per CTA of the plan's variant
-    int t_cta = 0;     // output samples computed per CTA (t_eff stored)
-    int t_eff = 0;     // output samples stored per CTA (tiles overlap)
+    int t_cta = 0;     // output samples computed per CTA (byte variants store 4 fewer: tiles overlap)
     int cb = 0;        // channels per shared-memory stage
     int win = 0;       // bytes per channel window in shared memory (the widest stage)
     int stages = 0;    // pipeline depth
@@ -221,6 +220,8 @@ cudaError_t launch_dedisperse_batch(const BeamLaunch *beams, int nbeams, int var
 cudaError_t launch_dedisperse_mma(const BeamLaunch *beams, int nbeams, bool add, int num_sms, int *err,
                                   cudaStream_t s, int32_t *nlaunch);
 int dedisperse_num_variants();
+// Smallest search block whose sums a variant accumulates.
+int dedisperse_min_block(int variant);
 // Variants the batch autotuner may time, in order of preference.
 int dedisperse_tune_candidates(const int **list);
 // Geometry of variant v for the largest in-block spreads (per DM-block size).
@@ -267,8 +268,8 @@ cudaError_t launch_dependent(void (*kern)(KArgs...), dim3 grid, dim3 block, size
     cfg.numAttrs = 1;
     return cudaLaunchKernelEx(&cfg, kern, args...);
 }
-gsp_status plan_prepare_search(gsp_plan_s *p, int64_t n_out, int32_t **D, int64_t *stride,
-                               unsigned long long **bsum);
+gsp_status plan_prepare_search(gsp_plan_s *p, int64_t n_out, int variant, int32_t **D,
+                               int64_t *stride, unsigned long long **bsum);
 gsp_status plan_check_input(gsp_plan_s *p, const uint8_t *x, int64_t n_in, int64_t x_stride,
                             int64_t *n_out);
 

@@ -126,3 +126,44 @@ def test_tensor_core_sums_to_24_bits(gsp, monkeypatch, nchan, values, descending
     gsp.gsp_search_series(plan, out, n_out)
     plain = gsp.gsp_search_stats(plan, n_out)
     assert (fused["sigma_b"] == plain["sigma_b"]).all() and (fused["bad"] == plain["bad"]).all()
+
+
+def test_autotuned_batch_with_short_blocks(gsp, monkeypatch):
+    """Plans on a byte variant whose batch is tuned to the tensor-core kernel, with search blocks
+    that the byte variant sums on the way and the tensor-core kernel does not."""
+    nchan, block, mma = 1024, 800, gsp.gsp_dedisperse_variants()[0] - 1
+    g = torch.Generator(device="cuda")
+    g.manual_seed(3)
+    plans, refs, xs, n_ins = [], [], [], []
+    for n_in, ndm in [(100000, 256), (90000, 240)]:
+        def make():
+            d, keep = gsp.make_desc(nchan, 1000.0, 1500.0, 49.152e-6, n_in, ndm=ndm, dm_step=0.25,
+                                    block_len=block, threshold=4.0)
+            return gsp.gsp_plan_create(d, keep)
+        monkeypatch.setenv("GSP_DD_VARIANT", "32")
+        plans.append(make())
+        assert gsp.gsp_dedisperse_variants(plans[-1])[1] == 32
+        monkeypatch.delenv("GSP_DD_VARIANT")
+        refs.append(make())
+        xs.append(torch.randint(0, 256, (nchan, (n_in + 15) // 16 * 16), dtype=torch.uint8,
+                                device="cuda", generator=g))
+        n_ins.append(n_in)
+    b = gsp.gsp_batch_create(plans, gsp.GSP_BATCH_PERSISTENT | gsp.GSP_BATCH_AUTOTUNE)
+    for _ in range(2):
+        gsp.gsp_batch_search(b, xs, n_ins)
+        got, n, st = gsp.gsp_batch_candidates(b)
+        assert st == gsp.GSP_OK and n > 0
+    assert mma in [v for v, _ in gsp.gsp_batch_tune_results(b)]
+    assert gsp.gsp_batch_info(b)[0] == mma   # 1.5 times faster than any byte variant here
+    off = 0
+    for i, (p, ref, x, n_in) in enumerate(zip(plans, refs, xs, n_ins)):
+        gsp.gsp_search(ref, x, n_in)
+        want, m, _ = gsp.gsp_candidates(ref)
+        mine = got[off:off + m]
+        off += m
+        assert (mine["beam"] == i).all()
+        for f in ("dm_idx", "t", "width", "snr"):
+            assert (mine[f] == want[f]).all(), (i, f)
+        n_out = gsp.gsp_plan_nout(p, n_in)
+        assert (gsp.gsp_search_stats(p, n_out)["sigma_b"] == gsp.gsp_search_stats(ref, n_out)["sigma_b"]).all()
+    assert off == n
