@@ -579,6 +579,7 @@ __global__ void __launch_bounds__(kThreads, 1) dd_mma_kernel(const __grid_consta
                         mma_ts(tmem, acol + (uint32_t)(k * 8), dlo + (uint32_t)(k * (kWidePitch / 16)), dhi,
                                idesc, (pos | k) != 0 ? 1u : 0u);
                     }
+                    if (!ok) break;
                     tc::mma_commit(empty);
                 }
                 if (!ok) break;

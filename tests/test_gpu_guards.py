@@ -167,3 +167,35 @@ def test_autotuned_batch_with_short_blocks(gsp, monkeypatch):
         n_out = gsp.gsp_plan_nout(p, n_in)
         assert (gsp.gsp_search_stats(p, n_out)["sigma_b"] == gsp.gsp_search_stats(ref, n_out)["sigma_b"]).all()
     assert off == n
+
+
+@pytest.mark.parametrize("cycles,starve", [(2_000_000, 1), (3000, 0), (1, 0)])
+def test_tensor_core_waits_that_run_out(gsp, monkeypatch, cycles, starve):
+    """Nothing copied, the row moves' wait for a frame of products too short, and every wait too
+    short: each comes back as a timeout, and the plan then gives exact sums."""
+    monkeypatch.setenv("GSP_DD_VARIANT", str(gsp.gsp_dedisperse_variants()[0] - 1))
+    nchan, n_in, ndm = 512, 100000, 40
+    d, keep = gsp.make_desc(nchan, 1200.0, 1500.0, 1e-4, n_in, ndm=ndm, dm_step=1.0)
+    plan = gsp.gsp_plan_create(d, keep)
+    assert gsp.gsp_dedisperse_variants(plan)[1] == gsp.gsp_dedisperse_variants()[0] - 1
+    g = torch.Generator(device="cuda")
+    g.manual_seed(4)
+    x = torch.randint(0, 256, (nchan, n_in), dtype=torch.uint8, device="cuda", generator=g)
+    dl = gsp.gsp_plan_delays(plan)
+    n_out = gsp.gsp_plan_nout(plan, n_in)
+    out = torch.zeros((ndm, (n_out + 3) // 4 * 4), dtype=torch.int32, device="cuda")
+    for _ in range(3):
+        gsp.gsp_plan_set_wait_limit(plan, cycles, starve)
+        gsp.gsp_search(plan, x, n_in, 0, out)
+        with pytest.raises(gsp.GspError) as e:
+            gsp.gsp_candidates(plan)
+        assert e.value.status == gsp.GSP_ERR_TIMEOUT
+        gsp.gsp_plan_set_wait_limit(plan, 4_000_000_000, 0)
+        gsp.gsp_search(plan, x, n_in, 0, out)
+        _, _, st = gsp.gsp_candidates(plan)
+        assert st == gsp.GSP_OK
+        for i in (0, 17, ndm - 1):
+            ref = torch.zeros(n_out, dtype=torch.int32, device="cuda")
+            for c in range(nchan):
+                ref += x[c, int(dl[i, c]):int(dl[i, c]) + n_out]
+            assert torch.equal(out[i, :n_out], ref), i
