@@ -510,9 +510,6 @@ gsp_status gsp_subband_create(gsp_subband_t *out, const gsp_plan_desc *desc, int
             off[(size_t)d * nsub + s] += b->min2[(size_t)(d / group) * nsub + s] & 3;
     if (e == cudaSuccess) e = cudaMemcpy(b->d_off2, off.data(), off.size() * 4, cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemset(b->d_err, 0, sizeof(int));
-    if (e == cudaSuccess && b->smem > 48 * 1024)
-        e = cudaFuncSetAttribute(subband_sum_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 b->smem);
     if (e != cudaSuccess) {
         gsp::record_error(e, "subband upload");
         free_subband(b);
@@ -585,12 +582,19 @@ gsp_status gsp_subband_dedisperse(gsp_subband_t b, const uint8_t *d_x, int64_t n
         }
     }
     // stage 2: sums of the sub-band series, shifted by the reference delays
+    // (the kernel's shared-memory limit is one for all sub-band objects of the process: it is
+    // only ever raised)
+    cudaError_t e = gsp::ensure_kernel_smem(reinterpret_cast<const void *>(subband_sum_kernel), b->smem);
+    if (e != cudaSuccess) {
+        gsp::record_error(e, "sub-band stage 2 attribute");
+        return GSP_ERR_CUDA;
+    }
     dim3 grid((unsigned)((n_out + kS2Tile - 1) / kS2Tile), (unsigned)b->nsdm);
     subband_sum_kernel<<<grid, (kS2Warps + 1) * 32, b->smem, s>>>(
         b->d_S, b->s_stride, b->nsdm, b->nsub, b->d_min2, b->d_off2, b->ndm, b->group, b->pitch,
         b->rows, b->stages, n_out, d_out, out_stride, b->d_err);
     b->launches += 1;
-    cudaError_t e = cudaGetLastError();
+    e = cudaGetLastError();
     if (e != cudaSuccess) {
         gsp::record_error(e, "sub-band stage 2 launch");
         return GSP_ERR_CUDA;

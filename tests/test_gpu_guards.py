@@ -199,3 +199,25 @@ def test_tensor_core_waits_that_run_out(gsp, monkeypatch, cycles, starve):
             for c in range(nchan):
                 ref += x[c, int(dl[i, c]):int(dl[i, c]) + n_out]
             assert torch.equal(out[i, :n_out], ref), i
+
+
+def test_sub_band_objects_side_by_side(gsp):
+    """Objects whose stage 2 needs different amounts of shared memory, used in turn."""
+    nchan, nsub, group, n_in = 64, 8, 16, 12000
+    x = torch.from_numpy(np.random.default_rng(6).integers(0, 256, (nchan, n_in), dtype=np.uint8)).cuda()
+    subs = []
+    for step in (4.0, 0.1, 1.0, 8.0):
+        d, keep = gsp.make_desc(nchan, 1200.0, 1500.0, 1e-4, n_in, ndm=32, dm_step=step)
+        subs.append(gsp.gsp_subband_create(d, nsub, group))
+    for sub in subs + subs:
+        d1, d2, _ = gsp.gsp_subband_delays(sub)
+        n = gsp.gsp_subband_nout(sub, n_in)
+        out = torch.full((32, (n + 3) // 4 * 4), -7, dtype=torch.int32, device="cuda")
+        gsp.gsp_subband_dedisperse(sub, x, n_in, out)
+        gsp.gsp_subband_finish(sub)
+        for k in (0, 31):
+            ref = torch.zeros(n, dtype=torch.int32, device="cuda")
+            for c in range(nchan):
+                o = int(d1[k // group, c] + d2[k, c // (nchan // nsub)])
+                ref += x[c, o:o + n]
+            assert torch.equal(out[k, :n], ref), k
