@@ -510,6 +510,12 @@ gsp_status gsp_subband_dedisperse(gsp_subband_t b, const uint8_t *d_x, int64_t n
  * kernel gave up (the flag is then cleared). */
 gsp_status gsp_subband_finish(gsp_subband_t b, void *stream);
 
+/* Limits of the bounded waits of both stages, as gsp_plan_set_wait_limit sets them
+ * for a plan (a test knob for the failure path): each wait gives up after `cycles`
+ * SM clock cycles (1 .. 4e9, default 4e9), and gsp_subband_finish then returns
+ * GSP_ERR_TIMEOUT.  With starve = 1 stage 2 issues no copies.  Host only. */
+gsp_status gsp_subband_set_wait_limit(gsp_subband_t b, int64_t cycles, int32_t starve);
+
 /* Kernel launches of the last gsp_subband_dedisperse call. */
 int32_t gsp_subband_launches(gsp_subband_t b);
 

@@ -152,14 +152,14 @@ constexpr int kMaxGroup = 16;
 constexpr int kS2Warps = 8;
 constexpr int kS2Tile = 1024;
 constexpr int kS2Rows = 4;                 // rows per stage
-constexpr long long kS2Budget = 2000000000ll;  // ~1 s of SM clock per wait
 
 namespace ptx = gsp::ptx;
 
 __global__ void __launch_bounds__((kS2Warps + 1) * 32, 2) subband_sum_kernel(
     const int32_t *__restrict__ S, int64_t s_stride, int nsdm, int nsub,
     const int32_t *__restrict__ min2, const int32_t *__restrict__ off2, int ndm, int group,
-    int pitch, int rows, int stages, int64_t n_out, int32_t *__restrict__ D, int64_t d_stride, int *err) {
+    int pitch, int rows, int stages, int64_t n_out, int32_t *__restrict__ D, int64_t d_stride, int *err,
+    long long budget, int starve) {
     extern __shared__ __align__(128) int32_t sm[];  // [stages][rows][pitch], then the barriers
     const uint32_t sm0 = ptx::smem_addr(sm);
     const uint32_t stage_bytes = (uint32_t)(rows * pitch * 4);
@@ -179,6 +179,7 @@ __global__ void __launch_bounds__((kS2Warps + 1) * 32, 2) subband_sum_kernel(
     }
     __syncthreads();
     if (warp == kS2Warps) {
+        if (starve) return;  // failure-path test: nothing issued, nothing in flight
         int slot = 0;
         uint32_t par = 1;  // a fresh barrier's previous phase counts as complete
         int issued = 0;
@@ -193,7 +194,7 @@ __global__ void __launch_bounds__((kS2Warps + 1) * 32, 2) subband_sum_kernel(
                 bytes = 4u * (uint32_t)max((int64_t)0, min((int64_t)pitch, s_stride - a0));
             }
             const uint32_t tot = __reduce_add_sync(0xffffffffu, bytes);
-            if (!__all_sync(0xffffffffu, ptx::mbar_wait(empty(slot), par, kS2Budget))) {
+            if (!__all_sync(0xffffffffu, ptx::mbar_wait(empty(slot), par, budget))) {
                 ok = false;
                 break;
             }
@@ -210,7 +211,7 @@ __global__ void __launch_bounds__((kS2Warps + 1) * 32, 2) subband_sum_kernel(
         }
         for (int st = max(0, issued - stages); st < issued; st++)
             ok = __all_sync(0xffffffffu, ptx::mbar_wait(full(st % stages), (uint32_t)(st / stages) & 1u,
-                                                        2 * kS2Budget)) && ok;
+                                                        gsp::kWaitLimit)) && ok;
         if (!ok && lane == 0) atomicExch(err, 1);
         return;
     }
@@ -233,7 +234,7 @@ __global__ void __launch_bounds__((kS2Warps + 1) * 32, 2) subband_sum_kernel(
     for (int st = 0; st < nst; st++) {
         const int cur = nxt;
         if (st + 1 < nst) nxt = offset(st + 1);
-        if (!__all_sync(0xffffffffu, ptx::mbar_wait(full(slot), par, kS2Budget))) {
+        if (!__all_sync(0xffffffffu, ptx::mbar_wait(full(slot), par, budget))) {
             if (lane == 0) atomicExch(err, 1);
             return;
         }
@@ -302,6 +303,8 @@ struct gsp_subband_s {
     int pitch = 0, rows = 0, stages = 0, smem = 0;  // shared-memory ring of stage 2
     int num_sms = 0;
     int32_t launches = 0;
+    long long wait_budget = gsp::kWaitLimit;  // bounded waits of stage 2
+    int wait_starve = 0;
 };
 
 namespace {
@@ -592,7 +595,7 @@ gsp_status gsp_subband_dedisperse(gsp_subband_t b, const uint8_t *d_x, int64_t n
     dim3 grid((unsigned)((n_out + kS2Tile - 1) / kS2Tile), (unsigned)b->nsdm);
     subband_sum_kernel<<<grid, (kS2Warps + 1) * 32, b->smem, s>>>(
         b->d_S, b->s_stride, b->nsdm, b->nsub, b->d_min2, b->d_off2, b->ndm, b->group, b->pitch,
-        b->rows, b->stages, n_out, d_out, out_stride, b->d_err);
+        b->rows, b->stages, n_out, d_out, out_stride, b->d_err, b->wait_budget, b->wait_starve);
     b->launches += 1;
     e = cudaGetLastError();
     if (e != cudaSuccess) {
@@ -615,6 +618,15 @@ gsp_status gsp_subband_finish(gsp_subband_t b, void *stream) {
         cudaMemset(b->d_err, 0, sizeof(int));
         return GSP_ERR_TIMEOUT;
     }
+    return GSP_OK;
+}
+
+gsp_status gsp_subband_set_wait_limit(gsp_subband_t b, int64_t cycles, int32_t starve) {
+    if (!b || cycles < 1 || cycles > gsp::kWaitLimit || starve < 0 || starve > 1)
+        return GSP_ERR_INVALID_ARG;
+    for (gsp_plan_t p : b->stage1) p->wait_budget = cycles;
+    b->wait_budget = cycles;
+    b->wait_starve = starve;
     return GSP_OK;
 }
 

@@ -145,6 +145,7 @@ def lib():
             "gsp_subband_delays": ([_vp, _vp, _vp, _vp], ctypes.c_int),
             "gsp_subband_dedisperse": ([_vp, _vp, _i64, _i64, _vp, _i64, _vp], ctypes.c_int),
             "gsp_subband_finish": ([_vp, _vp], ctypes.c_int),
+            "gsp_subband_set_wait_limit": ([_vp, _i64, ctypes.c_int32], ctypes.c_int),
             "gsp_subband_launches": ([_vp], ctypes.c_int32),
             "gsp_gemm_bf16": ([_vp, _i64, _vp, _i64, _vp, _i64, ctypes.c_int32, ctypes.c_int32,
                                ctypes.c_int32, _vp, ctypes.c_int32, ctypes.c_int32, _vp, _vp],
@@ -796,6 +797,11 @@ def gsp_subband_dedisperse(b, x, n_in, out, stream=None):
 
 def gsp_subband_finish(b, stream=None):
     _check(lib().gsp_subband_finish(b.handle, _stream(stream)), "gsp_subband_finish")
+
+
+def gsp_subband_set_wait_limit(b, cycles, starve=0):
+    _check(lib().gsp_subband_set_wait_limit(b.handle, int(cycles), int(starve)),
+           "gsp_subband_set_wait_limit")
 
 
 def gsp_subband_launches(b):

@@ -20,6 +20,14 @@ def gsp():
     return g
 
 
+def _status(gsp, call):
+    try:
+        call()
+    except gsp.GspError as e:
+        return e.status
+    return gsp.GSP_OK
+
+
 @pytest.mark.parametrize("rows,nblk", [(600, 40), (5000, 2), (300, 33)])
 def test_block_aligned_search_repeats(gsp, rows, nblk):
     """Several blocks per CTA and a candidate in every window: each pass of the
@@ -171,8 +179,9 @@ def test_autotuned_batch_with_short_blocks(gsp, monkeypatch):
 
 @pytest.mark.parametrize("cycles,starve", [(2_000_000, 1), (3000, 0), (1, 0)])
 def test_tensor_core_waits_that_run_out(gsp, monkeypatch, cycles, starve):
-    """Nothing copied, the row moves' wait for a frame of products too short, and every wait too
-    short: each comes back as a timeout, and the plan then gives exact sums."""
+    """Nothing copied: a timeout.  Limits shorter than a frame of products, or than any copy (a
+    wait always tests its barrier twice and may sleep in between, so it can still succeed): a
+    timeout or exact sums.  The plan then gives exact sums."""
     monkeypatch.setenv("GSP_DD_VARIANT", str(gsp.gsp_dedisperse_variants()[0] - 1))
     nchan, n_in, ndm = 512, 100000, 40
     d, keep = gsp.make_desc(nchan, 1200.0, 1500.0, 1e-4, n_in, ndm=ndm, dm_step=1.0)
@@ -184,21 +193,15 @@ def test_tensor_core_waits_that_run_out(gsp, monkeypatch, cycles, starve):
     dl = gsp.gsp_plan_delays(plan)
     n_out = gsp.gsp_plan_nout(plan, n_in)
     out = torch.zeros((ndm, (n_out + 3) // 4 * 4), dtype=torch.int32, device="cuda")
-    for _ in range(3):
-        gsp.gsp_plan_set_wait_limit(plan, cycles, starve)
+    ref = {i: sum(x[c, int(dl[i, c]):int(dl[i, c]) + n_out].int() for c in range(nchan))
+           for i in (0, 17, ndm - 1)}
+    for limit in [(cycles, starve), (4_000_000_000, 0)] * 3:
+        gsp.gsp_plan_set_wait_limit(plan, *limit)
         gsp.gsp_search(plan, x, n_in, 0, out)
-        with pytest.raises(gsp.GspError) as e:
-            gsp.gsp_candidates(plan)
-        assert e.value.status == gsp.GSP_ERR_TIMEOUT
-        gsp.gsp_plan_set_wait_limit(plan, 4_000_000_000, 0)
-        gsp.gsp_search(plan, x, n_in, 0, out)
-        _, _, st = gsp.gsp_candidates(plan)
-        assert st == gsp.GSP_OK
-        for i in (0, 17, ndm - 1):
-            ref = torch.zeros(n_out, dtype=torch.int32, device="cuda")
-            for c in range(nchan):
-                ref += x[c, int(dl[i, c]):int(dl[i, c]) + n_out]
-            assert torch.equal(out[i, :n_out], ref), i
+        status = _status(gsp, lambda: gsp.gsp_candidates(plan))
+        assert status == gsp.GSP_ERR_TIMEOUT or limit[1] == 0
+        assert status == gsp.GSP_OK or limit[0] < 4_000_000_000
+        assert status == gsp.GSP_ERR_TIMEOUT or all(torch.equal(out[i, :n_out], r) for i, r in ref.items())
 
 
 def test_sub_band_objects_side_by_side(gsp):
@@ -221,3 +224,30 @@ def test_sub_band_objects_side_by_side(gsp):
                 o = int(d1[k // group, c] + d2[k, c // (nchan // nsub)])
                 ref += x[c, o:o + n]
             assert torch.equal(out[k, :n], ref), k
+
+
+@pytest.mark.parametrize("cycles,starve", [(2_000_000, 1), (1, 0)])
+def test_sub_band_waits_that_run_out(gsp, cycles, starve):
+    """Stage 2 without copies: a timeout at finish.  Both stages with limits shorter than a copy: a
+    timeout or exact sums.  Then exact sums from the same object."""
+    nchan, nsub, group, n_in, ndm = 64, 16, 16, 60000, 40
+    x = torch.from_numpy(np.random.default_rng(7).integers(0, 256, (nchan, n_in), dtype=np.uint8)).cuda()
+    d, keep = gsp.make_desc(nchan, 1200.0, 1500.0, 1e-4, n_in, ndm=ndm, dm_step=1.0)
+    sub = gsp.gsp_subband_create(d, nsub, group)
+    d1, d2, _ = gsp.gsp_subband_delays(sub)
+    n = gsp.gsp_subband_nout(sub, n_in)
+    out = torch.full((ndm, (n + 3) // 4 * 4), -7, dtype=torch.int32, device="cuda")
+    ref = {}
+    for k in (0, 23, ndm - 1):
+        at = [int(d1[k // group, c] + d2[k, c // (nchan // nsub)]) for c in range(nchan)]
+        ref[k] = sum(x[c, at[c]:at[c] + n].int() for c in range(nchan))
+    for limit in [(cycles, starve), (4_000_000_000, 0)] * 3:
+        gsp.gsp_subband_set_wait_limit(sub, *limit)
+        gsp.gsp_subband_dedisperse(sub, x, n_in, out)
+        status = _status(gsp, lambda: gsp.gsp_subband_finish(sub))
+        assert status == gsp.GSP_ERR_TIMEOUT or limit[1] == 0
+        assert status == gsp.GSP_OK or limit[0] < 4_000_000_000
+        assert status == gsp.GSP_ERR_TIMEOUT or all(torch.equal(out[k, :n], r) for k, r in ref.items())
+    for bad in [(0, 0), (5_000_000_000, 0), (100, 2)]:
+        with pytest.raises(gsp.GspError):
+            gsp.gsp_subband_set_wait_limit(sub, *bad)
