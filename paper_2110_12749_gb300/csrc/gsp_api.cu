@@ -787,13 +787,21 @@ gsp_status gsp_plan_tune(gsp_plan_t p, const uint8_t *d_x, int64_t n_in, int64_t
     const int64_t stride = (n_out + 3) & ~(int64_t)3;
     const int *cand = nullptr;
     const int ncand = gsp::dedisperse_tune_candidates(&cand);
-    const int keep = p->geom.variant;
+    // a call that fails leaves the plan as it was, its rules for each launch included
+    struct Restore {
+        gsp_plan_s *plan;
+        gsp::DDGeom geom;
+        bool on = true;
+        ~Restore() {
+            if (on) plan->geom = geom;
+        }
+    } keep{p, p->geom};
     const bool split = p->geom.split;  // the plan's split between two kernels is timed too
     int best = -1;
     bool best_split = false;
     float best_t = 0.f;
     for (int ci = 0; ci < ncand + (split ? 1 : 0); ci++) {
-        const int v = ci < ncand ? cand[ci] : keep;
+        const int v = ci < ncand ? cand[ci] : keep.geom.variant;
         if (!gsp::dedisperse_variant_usable(p, v)) continue;
         gsp::dedisperse_set_variant(p, v);
         p->geom.split = ci == ncand;
@@ -804,8 +812,6 @@ gsp_status gsp_plan_tune(gsp_plan_t p, const uint8_t *d_x, int64_t n_in, int64_t
             cudaError_t e = gsp::launch_dedisperse_tiled(p, d_x, n + p->max_delay, x_stride, n,
                                                          p->d_D, stride, nullptr, s, &nl);
             if (e != cudaSuccess) {
-                gsp::dedisperse_set_variant(p, keep);
-                p->geom.split = split;
                 set_err(e, "tuning launch");
                 return GSP_ERR_CUDA;
             }
@@ -823,11 +829,14 @@ gsp_status gsp_plan_tune(gsp_plan_t p, const uint8_t *d_x, int64_t n_in, int64_t
             best_t = med;
         }
     }
-    gsp_status kst = take_kernel_error(p);
-    gsp::dedisperse_set_variant(p, best >= 0 ? best : keep);
-    p->geom.split = best >= 0 ? best_split : split;
-    if (kst != GSP_OK) return kst;
-    if (variant) *variant = p->geom.variant;
+    st = take_kernel_error(p);
+    if (st != GSP_OK) return st;
+    if (best >= 0) {
+        gsp::dedisperse_set_variant(p, best);
+        p->geom.split = best_split;
+        keep.on = false;
+    }
+    if (variant) *variant = best >= 0 ? best : keep.geom.variant;
     if (best_ms) *best_ms = best_t;
     return GSP_OK;
 }

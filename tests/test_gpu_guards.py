@@ -251,3 +251,28 @@ def test_sub_band_waits_that_run_out(gsp, cycles, starve):
     for bad in [(0, 0), (5_000_000_000, 0), (100, 2)]:
         with pytest.raises(gsp.GspError):
             gsp.gsp_subband_set_wait_limit(sub, *bad)
+
+
+def test_failed_tuning_leaves_the_plan(gsp, monkeypatch):
+    """A plan whose band is split between the two kernels: a tuning call whose launches time out
+    changes neither its variant nor the split."""
+    monkeypatch.delenv("GSP_DD_VARIANT", raising=False)
+    nchan, ndm, n_out = 1024, 240, 50001
+    base, _ = gsp.make_desc(nchan, 500.0, 3300.0, 98.304e-6, 1 << 20, ndm=ndm, dm_step=1.0)
+    n_in = n_out + int(gsp.gsp_compute_delays(base)[0].max())
+    d, keep = gsp.make_desc(nchan, 500.0, 3300.0, 98.304e-6, n_in, ndm=ndm, dm_step=1.0)
+    plan = gsp.gsp_plan_create(d, keep)
+    x = torch.randint(0, 256, (nchan, (n_in + 15) // 16 * 16), dtype=torch.uint8, device="cuda")
+    out = torch.zeros((ndm, (n_out + 3) // 4 * 4), dtype=torch.int32, device="cuda")
+    gsp.gsp_dedisperse(plan, x, n_in, out)
+    before, want = (gsp.gsp_dedisperse_variants(plan)[1], gsp.gsp_plan_launches(plan)), out.clone()
+    assert before[1] == 2
+    gsp.gsp_plan_set_wait_limit(plan, 1_000_000, 1)
+    assert _status(gsp, lambda: gsp.gsp_plan_tune(plan, x, n_in)) == gsp.GSP_ERR_TIMEOUT
+    gsp.gsp_plan_set_wait_limit(plan, 4_000_000_000, 0)
+    gsp.gsp_dedisperse(plan, x, n_in, out)
+    assert (gsp.gsp_dedisperse_variants(plan)[1], gsp.gsp_plan_launches(plan)) == before
+    assert torch.equal(out, want)
+    best, _ = gsp.gsp_plan_tune(plan, x, n_in)
+    gsp.gsp_dedisperse(plan, x, n_in, out)
+    assert gsp.gsp_dedisperse_variants(plan)[1] == best and torch.equal(out, want)
