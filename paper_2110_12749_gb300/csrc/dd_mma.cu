@@ -817,9 +817,10 @@ int mma_split(const int32_t *delays, int ndm, int C, bool rev, int step, double 
     size_t f = 0;
     double sum_r = 0.0;
     int at = 0;
-    for (int rest = (C - 1) / step * step; rest > 0; rest -= step) {
-        const int n = C - rest;
-        if (n > reach) break;
+    // the rest's rows start or end at the split, depending on the order: whole steps of them
+    // before it, or whole steps of positions
+    for (int n = rev && C % step ? C % step : step; n < std::min(C, reach + 1); n += step) {
+        const int rest = C - n;
         for (; at < n; at++) {
             while (f < frames.size() && frames[f].pos <= at) f++;
             sum_r += frames[f - 1].rmax;

@@ -40,9 +40,10 @@ struct MmaShape {
 // delays [ndm][C]; rev: positions run from the last channel to the first; the first
 // npos of them.  false: a block's delays drift apart by more than a tile.
 bool mma_plan_tables(const int32_t *delays, int ndm, int C, bool rev, int npos, MmaTables *t);
-// How many positions to take where the rest (a multiple of step channels) is left to a
-// kernel of other_rate additions per clock and SM and other_fixed clocks per sample of a
-// trial; 0 if that gains less than a twentieth.
+// How many positions to take where the rest is left to a kernel of other_rate additions
+// per clock and SM and other_fixed clocks per sample of a trial, which takes rows in whole
+// steps from the first on (the rest's first row, and its last one where more rows follow, is a
+// multiple of step); 0 if that gains less than a twentieth.
 int mma_split(const int32_t *delays, int ndm, int C, bool rev, int step, double other_rate,
               double other_fixed);
 // Longest tile (output samples) for a largest R.

@@ -1111,7 +1111,7 @@ bool plan_dedisperse_tiled(gsp_plan_s *p, TiledTables *tab) {
     // part, the byte kernel for the whole stages of steep channels before it (2048
     // channels, 500-3300 MHz, 3000 trials, 600011 samples: 26.7 -> 21.5 ms).
     if (!forced && !force_mma && variant != kMmaVariant) {
-        const int npos = mma_split(p->delays_h.data(), ndm, C, rev, 64, byte_rate(variant), byte_fixed(variant));
+        const int npos = mma_split(p->delays_h.data(), ndm, C, rev, kCbSizes[0], byte_rate(variant), byte_fixed(variant));
         if (npos > 0) {
             split = tables(npos) && mma_tile_len(p->mma.shape.rmax) >= kMmaMinTile;
             if (!split) tab->mma = MmaTables();
@@ -1296,12 +1296,11 @@ cudaError_t launch_dedisperse_batch(const BeamLaunch *beams, int nbeams, int var
             byte_launch_clocks(variant, C, ndm, n_out, num_sms)) {
             BeamLaunch steep = beams[0];
             steep.bsum = nullptr;
+            // whole stages of every byte variant (mma_split)
             const int c0 = p->desc.freq_descending ? n1 : 0, c1 = p->desc.freq_descending ? C : C - n1;
-            if (c0 % kVariants[variant].cb == 0 && (c1 == C || c1 % kVariants[variant].cb == 0)) {
-                cudaError_t e = launch_bytes(&steep, 1, variant, persistent, c0, c1, num_sms, err, s, nlaunch);
-                if (e != cudaSuccess) return e;
-                return launch_dedisperse_mma(beams, 1, true, num_sms, err, s, nlaunch);
-            }
+            cudaError_t e = launch_bytes(&steep, 1, variant, persistent, c0, c1, num_sms, err, s, nlaunch);
+            if (e != cudaSuccess) return e;
+            return launch_dedisperse_mma(beams, 1, true, num_sms, err, s, nlaunch);
         }
     }
     return launch_bytes(beams, nbeams, variant, persistent, 0, C, num_sms, err, s, nlaunch);

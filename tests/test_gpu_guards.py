@@ -276,3 +276,29 @@ def test_failed_tuning_leaves_the_plan(gsp, monkeypatch):
     best, _ = gsp.gsp_plan_tune(plan, x, n_in)
     gsp.gsp_dedisperse(plan, x, n_in, out)
     assert gsp.gsp_dedisperse_variants(plan)[1] == best and torch.equal(out, want)
+
+
+@pytest.mark.parametrize("nchan", [1000, 1023, 1030])
+@pytest.mark.parametrize("descending", [False, True])
+def test_band_split_in_both_orders(gsp, monkeypatch, nchan, descending):
+    """A wide band whose channel count is no whole number of stages is split between the two
+    kernels in either channel order, with the same sums as the byte kernel."""
+    ndm, n_out = 240, 50001
+    base, _ = gsp.make_desc(nchan, 500.0, 3300.0, 98.304e-6, 1 << 20, ndm=ndm, dm_step=1.0)
+    n_in = n_out + int(gsp.gsp_compute_delays(base)[0].max())
+    g = torch.Generator(device="cuda")
+    g.manual_seed(nchan)
+    x = torch.randint(0, 256, (nchan, (n_in + 15) // 16 * 16), dtype=torch.uint8, device="cuda", generator=g)
+    outs = []
+    for variant in (None, "42"):
+        if variant:
+            monkeypatch.setenv("GSP_DD_VARIANT", variant)
+        else:
+            monkeypatch.delenv("GSP_DD_VARIANT", raising=False)
+        d, keep = gsp.make_desc(nchan, 500.0, 3300.0, 98.304e-6, n_in, ndm=ndm, dm_step=1.0,
+                                freq_descending=descending)
+        plan = gsp.gsp_plan_create(d, keep)
+        outs.append(torch.zeros((ndm, (n_out + 3) // 4 * 4), dtype=torch.int32, device="cuda"))
+        gsp.gsp_dedisperse(plan, x, n_in, outs[-1])
+        assert gsp.gsp_plan_launches(plan) == (1 if variant else 2)
+    assert torch.equal(outs[0], outs[1])
