@@ -557,9 +557,7 @@ __global__ void __launch_bounds__(256, 3) boxcar_block_kernel(
     constexpr int B = kChunk, NW = kNumDefaultWidths;
     static_assert(B == 4 * kBoxThreads, "four samples per thread");
     __shared__ __align__(16) uint32_t sP[2][B + kTail];  // exclusive prefix sums of a block and the next
-    // warps' totals, by the parity of the block: the first two scans follow each other with
-    // no barrier between a warp's reads of the one and another's writes of the next
-    __shared__ uint32_t wtot[2][kBoxThreads / 32];
+    __shared__ uint32_t wtot[kBoxThreads / 32];  // warps' totals of the block being scanned
     __shared__ Peak wbest[kBoxThreads / 32];
     __shared__ float s_scale[NW];
     __shared__ int s_width[NW];
@@ -612,9 +610,9 @@ __global__ void __launch_bounds__(256, 3) boxcar_block_kernel(
                                                        : make_int4(0, 0, 0, 0);
     };
     // prefix sums of block u (loaded as v) into its buffer and behind block u - 1's.  The
-    // barrier in here separates this scan's writes of wtot from its reads, and the reads
-    // of scan(u - 1) from the writes of scan(u + 1), which use the same half; it also ends the
-    // search of block u - 2, whose buffer is rewritten, and its reads of wbest.
+    // barrier in here separates this scan's writes of wtot from its reads and ends the search of
+    // block u - 2, whose buffer is rewritten, and its reads of wbest; a barrier has to follow
+    // each scan before the next one writes wtot again.
     auto scan = [&](int u, const int4 &v, const BlockParam &q) {
         const uint32_t m = q.good ? ~0u : 0u;
         const uint32_t y0 = (uint32_t)(v.x - q.m) & m, y1 = (uint32_t)(v.y - q.m) & m;
@@ -626,12 +624,12 @@ __global__ void __launch_bounds__(256, 3) boxcar_block_kernel(
             const uint32_t a = __shfl_up_sync(0xffffffffu, incl, o);
             if (lane >= o) incl += a;
         }
-        if (lane == 31) wtot[u & 1][wid] = incl;
+        if (lane == 31) wtot[wid] = incl;
         __syncthreads();
         uint32_t pre = carry + incl - tot, all = 0;
 #pragma unroll
         for (int w = 0; w < kBoxThreads / 32; w++) {
-            const uint32_t a = wtot[u & 1][w];
+            const uint32_t a = wtot[w];
             pre += w < wid ? a : 0u;
             all += a;
         }
@@ -643,6 +641,7 @@ __global__ void __launch_bounds__(256, 3) boxcar_block_kernel(
 
     BlockParam q = bp[first];
     scan(first, load(first), q);
+    __syncthreads();  // not a half of wtot per block parity: 815 us against 799 at 500 x 250001
     int4 nv = load(first + 1);
     for (int u = first; u < last; u++) {
         const bool more = u + 1 < nb;  // the row goes on after this block
