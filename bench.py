@@ -27,13 +27,14 @@ ROOT = os.path.dirname(os.path.abspath(__file__))
 if ROOT not in sys.path:
     sys.path.insert(0, ROOT)
 
-# DRAM bytes (read + write) per algorithmic add of the byte kernel (variant 32): ncu
-# dram__bytes_read.sum + dram__bytes_write.sum of one launch on the CRAFTS-like beam
-# cut to 131072 samples (1.574 GB + 0.665 GB for 6.899e11 adds), the capture size
-# rule keeping full-size multi-pass captures off the GPU; traffic grows with the
-# number of time tiles, i.e. in proportion to the adds.
-DD_TRAFFIC_BYTES_PER_ADD = (1.5738e9 + 0.6653e9) / 6.899e11
-DD_TRAFFIC_VARIANT = 32
+# DRAM bytes (read + write) per algorithmic add: ncu dram__bytes_read.sum +
+# dram__bytes_write.sum of one launch on the CRAFTS-like beam cut to 131072 samples
+# (6.899e11 adds), the capture size rule keeping full-size multi-pass captures off the GPU;
+# traffic grows with the number of time tiles, i.e. in proportion to the adds.  The
+# tensor-core kernel, and variant 32 of the byte kernel.
+DD_TRAFFIC_TENSOR = (1.76e9 + 0.69e9) / 6.899e11
+DD_TRAFFIC_BYTE = (1.5738e9 + 0.6653e9) / 6.899e11
+DD_TRAFFIC_BYTE_VARIANT = 32
 
 NOMINAL_SMS = 152
 RANKER_KEYS = ("recall", "recall_nominal", "precision", "precision_snr8", "negatives_rejected", "threshold",
@@ -44,13 +45,18 @@ RANKER_KEYS = ("recall", "recall_nominal", "precision", "precision_snr8", "negat
 INT_LANES_PER_SM = 128          # issue slots per SM per clock (4 schedulers x 32 lanes)
 TENSOR_ADDS_PER_SM = 256        # additions per SM per clock of the tensor-core kernel: a K = 16
                                 # product (16 multiply-adds of 4096 per clock) does one
-TENSOR_VARIANT = 45             # index of that kernel among the dedispersion variants
 SM_MAX_MHZ = 2070.0
+
+
+def is_tensor(variant):
+    """Whether a dedispersion variant is the tensor-core kernel (the last index)."""
+    from paper_2110_12749_gb300 import gsp
+    return variant == gsp.gsp_dedisperse_variants()[0] - 1
 
 
 def dd_peak(nsm, variant):
     """Peak of a dedispersion variant in T additions per second (maximum SM clock)."""
-    per_sm = TENSOR_ADDS_PER_SM if variant == TENSOR_VARIANT else INT_LANES_PER_SM
+    per_sm = TENSOR_ADDS_PER_SM if is_tensor(variant) else INT_LANES_PER_SM
     return nsm * per_sm * SM_MAX_MHZ * 1e6 / 1e12
 
 
@@ -837,8 +843,10 @@ def run_gsp(args):
     nsm = torch.cuda.get_device_properties(local).multi_processor_count
     clocks = clk.summary()
     dd_used = gsp.gsp_dedisperse_variants(plan)[1]
-    dd_tensor = dd_used == TENSOR_VARIANT
+    dd_tensor = is_tensor(dd_used)
     peak = dd_peak(nsm, dd_used)
+    dd_traffic = (DD_TRAFFIC_TENSOR if dd_tensor else
+                  DD_TRAFFIC_BYTE if dd_used == DD_TRAFFIC_BYTE_VARIANT else None)
     line = None
     stream_res = None
     batch_res = None
@@ -885,7 +893,7 @@ def run_gsp(args):
             "kernel_ms": {"dedisperse": dd_avg, "search": sum(se_ms) / len(se_ms)},
             "roofline": {"bound": "tensor" if dd_tensor else "alu", "achieved": achieved, "peak": peak, "unit": "Tadd/s",
                          "frac": achieved / peak,
-                         "traffic": (DD_TRAFFIC_BYTES_PER_ADD * adds if dd_used == DD_TRAFFIC_VARIANT else None),
+                         "traffic": dd_traffic * adds if dd_traffic else None,
                          "peak_basis": "%d SMs x %d %s x %.0f MHz (max clock)"
                                        % (nsm, TENSOR_ADDS_PER_SM if dd_tensor else INT_LANES_PER_SM,
                                           "adds of a K = 16 product" if dd_tensor else "int lanes", SM_MAX_MHZ),
