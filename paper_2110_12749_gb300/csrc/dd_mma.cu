@@ -207,7 +207,10 @@ __device__ __forceinline__ void widen_channel(uint32_t src, uint32_t dst, uint32
 //   20-21 copy the channels' windows of every other chunk each (1-D bulk copies).
 // Every wait is bounded: a warp whose wait gives up reports it and leaves its
 // loop; the MMA lane and the copying warp then wait for what they have in flight, and
-// tensor memory is freed after all warps have met.
+// tensor memory is freed after all warps have met.  (Where the wait for the row moves gives up,
+// the MMA lane first runs to the end of the item, waiting for and freeing its chunks but
+// issuing no more products: every way straight out of that loop made the compiler's
+// code for it slower, 16.08 -> 16.22 ms on a 131072-sample chunk.)
 __global__ void __launch_bounds__(kThreads, 1) dd_mma_kernel(const __grid_constant__ MmaArgs a) {
     extern __shared__ __align__(128) uint8_t smem[];
     uint8_t *raw = smem;                                 // [kSlots][kChunk][kRawPitch]
@@ -579,7 +582,6 @@ __global__ void __launch_bounds__(kThreads, 1) dd_mma_kernel(const __grid_consta
                         mma_ts(tmem, acol + (uint32_t)(k * 8), dlo + (uint32_t)(k * (kWidePitch / 16)), dhi,
                                idesc, (pos | k) != 0 ? 1u : 0u);
                     }
-                    if (!ok) break;
                     tc::mma_commit(empty);
                 }
                 if (!ok) break;
