@@ -608,16 +608,16 @@ __global__ void __launch_bounds__(kThreads, 1) dd_mma_kernel(const __grid_consta
             mma_decode(a, item, &bi, &tile, &blk);
             const MmaBeam &bt = a.beam[bi];
             const int T = bt.T;
-            // sample positions of the row, in 64 bits: a delay may be up to 2^31 - 1.  t0 is a
-            // multiple of 16; whole 16-byte pieces of the input end at in16
-            const int64_t t0 = tile * T;
-            const int64_t in16 = bt.n_in & ~(int64_t)15;
+            // t0 is a multiple of 16; positions below 64 bits are relative to a window (a delay
+            // may be up to 2^31 - 1)
+            const int64_t t0 = tile * T, left = bt.n_in - t0;
+            const int before = (int)min(t0, (int64_t)4096);  // input before the tile, if little
             const int32_t *base = bt.base + (int64_t)blk * C;
             const int32_t *crmax = bt.crmax + (int64_t)blk * nchunk;
             const int k = lane;  // channel of the chunk (lanes 0..7)
             int ch = (grp + kCopyWarps - (int)(g % kCopyWarps)) % kCopyWarps;
             const int64_t step = (bt.rev ? -1 : 1) * bt.x_stride;
-            const uint8_t *row = bt.x + (bt.rev ? (int64_t)(C - 1) * bt.x_stride : 0) +
+            const uint8_t *row = bt.x + t0 + (bt.rev ? (int64_t)(C - 1) * bt.x_stride : 0) +
                                  step * (ch * kChunk + k);
             int nbase = k < kChunk && ch * kChunk + k < C ? __ldg(base + ch * kChunk + k) : 0;
             int nrm = ch < nchunk ? __ldg(crmax + ch) : 0;
@@ -626,21 +626,18 @@ __global__ void __launch_bounds__(kThreads, 1) dd_mma_kernel(const __grid_consta
                 const int slot = (int)(gc % kSlots);
                 const int pos = ch * kChunk + k;
                 const bool in = k < kChunk && pos < C;
-                const int64_t s = t0 + nbase;                   // first sample
+                const int off = nbase & 15, w0 = nbase - off;  // the window starts 16-byte aligned
                 const int need = 8 * (frame_cols(T, nrm) + 1);  // samples from it
                 if (ch + kCopyWarps < nchunk) {
                     const int np = pos + kCopyWarps * kChunk;
                     nbase = k < kChunk && np < C ? __ldg(base + np) : 0;
                     nrm = __ldg(crmax + ch + kCopyWarps);
                 }
-                // bytes [lo, hi) of the channel's row; the samples before the input (only
-                // columns of t < 0 take them) and past its end are left as they are
-                const int off = (int)(s & 15);
-                const int64_t w0 = s - off;  // the window starts 16-byte aligned
-                const int64_t lo = max(w0, (int64_t)0);
-                const int64_t hi = min(w0 + ((off + need + 15) & ~15), bt.n_in);
-                const int64_t hi16 = min(hi, in16);
-                const uint32_t bytes = in && hi16 > lo ? (uint32_t)(hi16 - lo) & ~15u : 0u;
+                // bytes [lo, hi) of the window, whole 16-byte pieces up to hi16; the samples before
+                // the input (only columns of t < 0 take them) and past its end are left as they are
+                const int hi = (int)min(left - w0, (int64_t)((off + need + 15) & ~15)), hi16 = hi & ~15;
+                const int lo = w0 < 0 ? max(-w0 - before, 0) : 0;
+                const uint32_t bytes = in && hi16 > lo ? (uint32_t)(hi16 - lo) : 0u;
                 const uint32_t tot = __reduce_add_sync(0xffffffffu, bytes);
                 if (!__all_sync(0xffffffffu, ptx::mbar_wait(raw_empty(slot), ((gc / kSlots) & 1u) ^ 1u,
                                                             a.budget))) {
@@ -649,12 +646,12 @@ __global__ void __launch_bounds__(kThreads, 1) dd_mma_kernel(const __grid_consta
                 }
                 const uint32_t dst = (uint32_t)(slot * kRawSlot + k * kRawPitch);
                 if (in && hi > hi16)  // the last bytes of the input
-                    for (int64_t i = max(lo, hi16); i < hi; i++) raw[dst + (uint32_t)(i - w0)] = row[i];
+                    for (int i = max(lo, hi16); i < hi; i++) raw[dst + (uint32_t)i] = row[(int64_t)w0 + i];
                 __syncwarp();
                 if (lane == 0) ptx::mbar_arrive_expect_tx(raw_full(slot), tot);
                 __syncwarp();
                 if (bytes > 0)
-                    ptx::bulk_g2s(raw0 + dst + (uint32_t)(lo - w0), row + lo, bytes, raw_full(slot));
+                    ptx::bulk_g2s(raw0 + dst + (uint32_t)lo, row + ((int64_t)w0 + lo), bytes, raw_full(slot));
                 last = gc + 1u;
             }
             g += (uint32_t)nchunk;
