@@ -600,7 +600,8 @@ gsp_status gsp_ranker_forward(gsp_ranker_t r, const float *d_x, int32_t n, float
 /* One training step on n snippets with labels d_labels (device int32, 0 or
  * 1): forward, gradients of the mean cross-entropy, one Adam update with
  * learning rate lr.  d_loss (device float, optional) receives the batch loss.
- * Asynchronous. */
+ * Weight and bias gradients are FP32 sums added atomically from many blocks, so that
+ * their last bits may differ from run to run.  Asynchronous. */
 gsp_status gsp_ranker_train_step(gsp_ranker_t r, const float *d_x, const int32_t *d_labels,
                                  int32_t n, float lr, float *d_loss, void *stream);
 

@@ -27,12 +27,12 @@
 // the block; between frames row group i is moved right by e_i = 0..16 samples
 // inside tensor memory (a lane rotation within the 8 phases and a move by up
 // to two columns).  A frame is centred on a channel ahead of its first one, so it
-// spans twice the 8 samples: some 30 frames for the 4096 channels at a DM step
-// of 0.5, 1000-1500 MHz.
+// spans twice the 8 samples: 22 frames for the 4096 channels at a DM step of 0.5,
+// 1000-1500 MHz, 36 at 0.8.
 //
 // Bound.  Per channel and block an MMA issues 128 x N x 16 products for 128 N
-// useful additions and takes N / 2 clocks of the tensor pipe (136 measured at
-// N = 256, alone): 256 additions per clock and SM, against 86 of the shared-load bound
+// useful additions and takes N / 2 clocks of the tensor pipe (measured: 120 at N = 240,
+// 136 at N = 256): 256 additions per clock and SM, against 86 of the shared-load bound
 // kernel in dedisperse.cu.  The same 16 x N samples are copied, widened
 // and read from shared memory: 2 (copy) + 3 + 4 (widen) + 8 (operand) bytes per
 // 8 samples x 128-byte clock, which nearly fills the shared-memory port too.
@@ -841,14 +841,15 @@ int mma_split(const int32_t *delays, int ndm, int C, bool rev, int step, double 
 
 int mma_tile_len(int rmax) { return std::max(0, (8 * kCols - rmax) & ~15); }
 
-// Measured on GB300: 165 clocks per channel at T + R = 1840 samples (the product alone
-// takes 115; the rest is the shared-memory port's, see above) and not under 152 for a
-// shorter tile, 5,500 per frame boundary (drain, move, restart), 13,000 per item for the
-// epilogue, 8 per sample for reading the series that it adds to (17 without the lines
-// fetched ahead: 842 channels, 2062 trials 2046 us, 1956 with).  Within 4% of 25
-// launches of 325 to 3700 channels and 3 to 67 waves; the same without the floor and
-// with 4,000 per boundary was up to 40% low, and took grids of step 0.75 at 1000-1300
-// channels (2.50 ms) from the byte kernel (2.23).
+// Measured on GB300: 165 clocks per channel at T + R = 1840 samples (the product, N = 240,
+// takes 120; the rest is the shared-memory port's, see above) and not under 152 for a
+// shorter tile, 5,500 per frame boundary (drain, move, restart), 14,000 per item for its
+// start and epilogue, 8 per sample for reading the series that it adds to (17 without the
+// lines fetched ahead: 842 channels, 2062 trials 2046 us, 1956 with).  Within 4% of 23 out of
+// 26 launches of 74 to 4096 channels, 6 and 12% high at 74 channels and 5% at 664; the choice
+// by it was within 2% of the fastest kernel but at 74 channels (3 and 7%, between two
+// byte variants).  The same without the floor and with 4,000 per boundary was up to 40% low,
+// and took grids of step 0.75 at 1000-1300 channels (2.50 ms) from the byte kernel (2.23).
 double mma_item_clocks(const MmaShape &m, int nchan, int T, bool add) {
     return nchan * std::max(152.0, 0.67 * ((T + m.mean_r) / 8.0 + 8.0) + 4.0) +
            m.frames_per_block * (14.0 * T / 8.0 + 2900.0) + 14000.0 + (add ? 8.0 * T : 0.0);

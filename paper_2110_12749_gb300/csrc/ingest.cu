@@ -64,7 +64,8 @@ __global__ void __launch_bounds__(256) ingest_transpose_kernel(const uint8_t *__
 // The tile's word column is XORed with 8 times the channel group, which keeps both
 // sides free of bank conflicts.  About 1.1 instructions per byte (four when each
 // byte was gathered from shared memory on its own).  4096 x 262144 samples: 466 -> 349 us
-// with nothing of them in L2 (6.2 TB/s of the 6.8 measured).  Edge tiles fall back to byte accesses.
+// with nothing of them in L2, 320 with the order of tiles below (6.7 TB/s of the 6.8 measured).
+// Edge tiles fall back to byte accesses.
 // kVec: the input pointer and stride are 16-byte aligned too, and a thread's 16 bytes
 // are one load.  Otherwise they are five aligned words shifted into place, where those
 // words lie inside the matrix, or bytes (706 x 110948 samples with rows of 710 bytes:

@@ -46,6 +46,7 @@ __host__ __device__ constexpr int side_of(int l) { return l == 0 ? 64 : (l == 1 
 __host__ __device__ constexpr int round8(int v) { return (v + 7) & ~7; }
 __host__ __device__ constexpr int kdim(int l) { return 9 * cin_of(l); }         // im2col K
 __host__ __device__ constexpr int kpad(int l) { return round8(kdim(l)); }
+constexpr int kSms = 152;      // SMs of a GB300: loops over the grid are sized for them
 constexpr int kGradRows = 16;  // rows of the input-gradient weights (at least Cin of layers 1, 2)
 
 // Parameter offsets in the flat FP32 vector (order w1 b1 w2 b2 w3 b3 w4 b4 w5 b5,
@@ -943,7 +944,7 @@ void free_ranker(gsp_ranker_s *r) {
 }
 
 int blocks_for(int64_t n, int threads = 256) {
-    return (int)std::min<int64_t>((n + threads - 1) / threads, 152 * 16);
+    return (int)std::min<int64_t>((n + threads - 1) / threads, kSms * 16);
 }
 
 #define RK_LAUNCH(...)                                \
@@ -1030,7 +1031,7 @@ cudaError_t forward(gsp_ranker_s *r, const float *x, int n, bool train, cudaStre
     const float *const b1 = r->params + r->off.b[1], *const b2 = r->params + r->off.b[2];
     cudaError_t e;
     if (train) {
-        RK_LAUNCH((conv0_train_tc_kernel<<<(int)std::min<int64_t>((int64_t)n * kS * kS / 128, 152 * 16), 128, 0,
+        RK_LAUNCH((conv0_train_tc_kernel<<<(int)std::min<int64_t>((int64_t)n * kS * kS / 128, kSms * 16), 128, 0,
                                            s>>>(x, n, r->W[0], r->params + r->off.b[0], r->a[0], r->z[0],
                                                 r->idx[0], r->err)));
         e = launch_conv<8, 16, 32, kTrain>(r, r->a[0], n, r->W[1], b1, r->a[1], r->z[1], r->idx[1], 0, s);
@@ -1046,7 +1047,7 @@ cudaError_t forward(gsp_ranker_s *r, const float *x, int n, bool train, cudaStre
     // fc1 (K = 2048) as a deterministic split-K product: enough K chunks for a
     // CTA per SM even at one column block, at least four 64-wide steps each;
     // the chunks' partial products are summed in order by fc1_finish_kernel
-    int dev = 0, nsm = 152;
+    int dev = 0, nsm = kSms;
     if (cudaGetDevice(&dev) == cudaSuccess)
         (void)cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
     const int mt = (n + 127) / 128;
@@ -1085,7 +1086,7 @@ cudaError_t backward(gsp_ranker_s *r, const float *x, const int32_t *labels, int
     float *const gr = r->grads;
     const Offsets &o = r->off;
     RK_LAUNCH((loss_kernel<<<1, 256, 0, s>>>(r->z5, labels, n, r->g5, r->loss)));
-    RK_LAUNCH((fc2_back_kernel<<<std::min((n + 3) / 4, 152), kHid, 0, s>>>(
+    RK_LAUNCH((fc2_back_kernel<<<std::min((n + 3) / 4, kSms), kHid, 0, s>>>(
         r->g5, r->a4, r->params + o.w[4], r->z4, n, gr + o.w[4], gr + o.b[4], r->g4, r->g4T, n8,
         gr + o.b[3])));
     {
@@ -1102,17 +1103,17 @@ cudaError_t backward(gsp_ranker_s *r, const float *x, const int32_t *labels, int
         r->ga[2], r->idx[2], r->a[2], n, 16, r->gz[2], gr + o.b[2])));
     e = launch_conv<32, kGradRows, 16, kGrad>(r, r->gz[2], n, r->WG[2], nullptr, nullptr, r->ga[1], nullptr, 16, s);
     if (e != cudaSuccess) return e;
-    RK_LAUNCH((conv_dw_kernel<bf16, 16, 32, 16><<<std::min(n, 912), 256, 0, s>>>(
+    RK_LAUNCH((conv_dw_kernel<bf16, 16, 32, 16><<<std::min(n, 6 * kSms), 256, 0, s>>>(
         r->a[1], n, r->ga[2], r->idx[2], r->a[2], gr + o.w[2])));
     RK_LAUNCH((pool_back_kernel<16><<<blocks_for((int64_t)n * 16 * 16 * 2), 256, 0, s>>>(
         r->ga[1], r->idx[1], r->a[1], n, 32, r->gz[1], gr + o.b[1])));
     e = launch_conv<16, kGradRows, 32, kGrad>(r, r->gz[1], n, r->WG[1], nullptr, nullptr, r->ga[0], nullptr, 8, s);
     if (e != cudaSuccess) return e;
-    RK_LAUNCH((conv_dw_kernel<bf16, 8, 16, 32><<<std::min(2 * n, 912), 256, 0, s>>>(
+    RK_LAUNCH((conv_dw_kernel<bf16, 8, 16, 32><<<std::min(2 * n, 6 * kSms), 256, 0, s>>>(
         r->a[0], n, r->ga[1], r->idx[1], r->a[1], gr + o.w[1])));
     RK_LAUNCH((pool_back_kernel<8><<<blocks_for((int64_t)n * 32 * 32), 256, 0, s>>>(
         r->ga[0], r->idx[0], r->a[0], n, 64, r->gz[0], gr + o.b[0])));
-    RK_LAUNCH((conv_dw_kernel<float, 1, 8, 64><<<std::min(4 * n, 912), 256, 0, s>>>(
+    RK_LAUNCH((conv_dw_kernel<float, 1, 8, 64><<<std::min(4 * n, 6 * kSms), 256, 0, s>>>(
         x, n, r->ga[0], r->idx[0], r->a[0], gr + o.w[0])));
     r->step++;
     const double c1 = 1.0 - std::pow(0.9, (double)r->step);
