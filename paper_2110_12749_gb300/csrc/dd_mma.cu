@@ -912,7 +912,7 @@ cudaError_t launch_dedisperse_mma(const BeamLaunch *beams, int nbeams, bool add,
         bt.ndm = p->desc.ndm;
         bt.nblk = (p->desc.ndm + kKdm - 1) / kKdm;
         bt.grp = p->geom.grp[kdm_index(kKdm)];
-        if (in.bsum && bt.B < kMmaMinBlock) return cudaErrorInvalidValue;
+        if (in.bsum && (bt.B < kMmaMinBlock || bt.B > kMmaMaxBlock)) return cudaErrorInvalidValue;
         // the longest tiles for a batch, those of the best wave count for one beam
         const int tmax = mma_tile_len(p->mma.shape.rmax);
         if (tmax < 16) return cudaErrorInvalidValue;

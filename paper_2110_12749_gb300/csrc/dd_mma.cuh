@@ -8,6 +8,7 @@ namespace gsp {
 
 constexpr int kMmaMaxBeams = 32;    // beams per launch
 constexpr int kMmaMinBlock = 1024;  // smallest search block whose sums the kernel accumulates
+constexpr int kMmaMaxBlock = 1 << 30;  // and the largest: a tile's block ends stay within 32 bits
 
 // A run of channels (positions pos .. the next frame's pos, in order of
 // increasing delay) whose rows keep their displacement R; e: how far each row

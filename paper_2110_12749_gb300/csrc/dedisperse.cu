@@ -1125,8 +1125,9 @@ bool plan_dedisperse_tiled(gsp_plan_s *p, TiledTables *tab) {
 
 int dedisperse_num_variants() { return kNumVariants + 1; }
 
-int dedisperse_min_block(int variant) {
-    return variant == kMmaVariant ? kMmaMinBlock : 128 * kVariants[variant].m - 4;
+bool dedisperse_sums_blocks(int variant, int block_len) {
+    if (variant == kMmaVariant) return block_len >= kMmaMinBlock && block_len <= kMmaMaxBlock;
+    return block_len >= 128 * kVariants[variant].m - 4;
 }
 
 int dedisperse_tune_candidates(const int **list) {
@@ -1288,7 +1289,7 @@ cudaError_t launch_dedisperse_batch(const BeamLaunch *beams, int nbeams, int var
             return launch_dedisperse_mma(beams, nbeams, false, num_sms, err, s, nlaunch);
         variant = bv;
     } else if (nbeams == 1 && p->geom.split && variant == p->geom.variant &&
-               (!beams[0].bsum || p->desc.block_len >= kMmaMinBlock)) {
+               (!beams[0].bsum || dedisperse_sums_blocks(kMmaVariant, p->desc.block_len))) {
         // the steep channels' sums first, then the others' added to them
         const int n1 = p->mma.shape.npos;
         if (mma_launch_clocks(p->mma.shape, n1, ndm, n_out, num_sms, true, &T) +

@@ -201,10 +201,10 @@ gsp_status ensure_scratch_D(gsp_plan_s *p, int64_t n_out) {
 
 // Block sums are fused into the dedispersion kernel when the variant that is launched
 // can produce them: search blocks at least as long as a byte variant's tile (which then
-// touches at most two of them), or as the tensor-core kernel's smallest block.
+// touches at most two of them), or within the tensor-core kernel's limits.
 bool fused_stats(const gsp_plan_s *p, int variant) {
     return !p->simple_dd && p->d_bsum != nullptr &&
-           p->desc.block_len >= gsp::dedisperse_min_block(variant);
+           gsp::dedisperse_sums_blocks(variant, p->desc.block_len);
 }
 
 gsp_status run_dedisperse(gsp_plan_s *p, const uint8_t *x, int64_t n_in, int64_t x_stride,

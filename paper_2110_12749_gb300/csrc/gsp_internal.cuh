@@ -220,8 +220,8 @@ cudaError_t launch_dedisperse_batch(const BeamLaunch *beams, int nbeams, int var
 cudaError_t launch_dedisperse_mma(const BeamLaunch *beams, int nbeams, bool add, int num_sms, int *err,
                                   cudaStream_t s, int32_t *nlaunch);
 int dedisperse_num_variants();
-// Smallest search block whose sums a variant accumulates.
-int dedisperse_min_block(int variant);
+// Whether a variant accumulates the sums of search blocks of this length.
+bool dedisperse_sums_blocks(int variant, int block_len);
 // Variants the batch autotuner may time, in order of preference.
 int dedisperse_tune_candidates(const int **list);
 // Geometry of variant v for the largest in-block spreads (per DM-block size).

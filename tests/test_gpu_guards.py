@@ -302,3 +302,21 @@ def test_band_split_in_both_orders(gsp, monkeypatch, nchan, descending):
         gsp.gsp_dedisperse(plan, x, n_in, outs[-1])
         assert gsp.gsp_plan_launches(plan) == (1 if variant else 2)
     assert torch.equal(outs[0], outs[1])
+
+
+@pytest.mark.parametrize("block_len", [1 << 20, (1 << 30) + 16, (1 << 31) - 1])
+def test_search_blocks_longer_than_the_series(gsp, monkeypatch, block_len):
+    """Search blocks up to the longest that a plan accepts, on the tensor-core kernel: no whole
+    block, so no candidates, and the same series."""
+    monkeypatch.setenv("GSP_DD_VARIANT", str(gsp.gsp_dedisperse_variants()[0] - 1))
+    nchan, n_in, ndm = 40, 30000, 20
+    d, keep = gsp.make_desc(nchan, 1200.0, 1500.0, 1e-4, n_in, ndm=ndm, dm_step=1.0, block_len=block_len)
+    plan = gsp.gsp_plan_create(d, keep)
+    x = torch.from_numpy(np.random.default_rng(9).integers(0, 256, (nchan, (n_in + 15) // 16 * 16), dtype=np.uint8)).cuda()
+    dl, n_out = gsp.gsp_plan_delays(plan), gsp.gsp_plan_nout(plan, n_in)
+    out = torch.zeros((ndm, (n_out + 3) // 4 * 4), dtype=torch.int32, device="cuda")
+    gsp.gsp_search(plan, x, n_in, 0, out)
+    c, n, st = gsp.gsp_candidates(plan)
+    assert n == 0 and st == gsp.GSP_OK
+    ref = sum(x[k, int(dl[ndm - 1, k]):int(dl[ndm - 1, k]) + n_out].int() for k in range(nchan))
+    assert torch.equal(out[ndm - 1, :n_out], ref)
